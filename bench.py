@@ -169,7 +169,7 @@ KERNEL_SOURCES = {
                                "mot_internal.h"],
     "umma2_wide_translate": ["wide.cu", "umma_common.cuh", "gelu.cuh", "ptx.cuh", "mot_internal.h"],
     # replay stages: guided attention, selection (with the SIMT kernels), full attention
-    "replay_attn_sparse": ["replay_gattn.cu", "replay_common.cuh", "replay_internal.h",
+    "replay_attn_sparse": ["replay_gather.cu", "replay_common.cuh", "replay_internal.h",
                            "mot_internal.h", "ptx.cuh"],
     "replay_select": ["replay.cu", "replay_common.cuh", "replay_internal.h", "mot_internal.h",
                       "ptx.cuh"],

@@ -231,9 +231,9 @@ mot_status mot_profile_read(mot_handle h, mot_kernel_stat* out, int32_t cap, int
  * first CTA of the single-SM GEMM1 kernel (schedule 0) never fills its first
  * pipeline stage, so a wait on it runs out: translations then report
  * MOT_ERR_TIMEOUT through mot_get_device_status and the context stays usable.
- * On a replay handle, stall_test = 1 makes the tensor-core guided attention's
- * first CTA withhold the completion signal of its first MMA, with the same
- * outcome for mot_replay_attention on a guided layer.
+ * On a replay handle, stall_test = 1 makes the guided attention's first CTA
+ * wait for a signal that nothing sends, with the same outcome for
+ * mot_replay_attention on a guided layer.
  */
 mot_status mot_debug_set(mot_handle h, int32_t stall_test, int64_t wait_limit_cycles);
 
@@ -415,9 +415,9 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
  * j <= u is read; guide may be NULL for full layers). Rows u >= seq_lens[b] of
  * out are not written. seq_lens: device int32[batch], clamped to [0, max_seq].
  * Requires head_dim in {64, 128}, q_heads / kv_heads in 1..8, 12 or 16, top_s <= 4096,
- * max_seq <= 65536 (else MOT_ERR_UNSUPPORTED). Asynchronous on `stream`. Guided
- * layers with head_dim 128 and top_s <= 128 run on the tensor cores, full
- * layers with max_seq % 8 == 0 too; other shapes take the SIMT kernels.
+ * max_seq <= 65536 (else MOT_ERR_UNSUPPORTED). Asynchronous on `stream`. Full
+ * layers with max_seq % 8 == 0 run the tiled causal kernel; guided layers and
+ * the other full layers attend row by row over gathered keys and values.
  *
  * mot_replay_select writes the selection alone: sel [max_batch][max_seq][top_s]
  * int32, the row's positions ascending, then -1 (rows u >= seq_lens[b] are not

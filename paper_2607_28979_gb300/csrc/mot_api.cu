@@ -188,6 +188,12 @@ struct mot_ctx {
 
 namespace {
 
+// Entries per row of the replay selection workspace: top_s in whole units of the attention.
+int64_t sel_row(const ReplayDims& d) {
+  const int64_t unit = replay_gather_unit(d);
+  return (int64_t(d.S) + unit - 1) / unit * unit;
+}
+
 size_t esize(const Dims& d) { return d.dtype == 0 ? 2 : 4; }
 size_t src_bytes(const Dims& d) {
   return size_t(d.L_s) * d.B * d.H_s * size_t(d.S) * d.d_s * esize(d);
@@ -1543,7 +1549,7 @@ mot_status mot_create_replay(const mot_replay_config* cfg, mot_handle* out) {
     return MOT_ERR_UNSUPPORTED;
   }
   const size_t vt_bytes = replay_fmha_supported(rd) ? size_t(rd.B) * rd.Hkv * rd.d * rd.N * 2 : 16;
-  if (cudaMalloc(&h->rsel, size_t(rd.B) * rd.N * rd.S * 4) != cudaSuccess ||
+  if (cudaMalloc(&h->rsel, size_t(rd.B) * rd.N * sel_row(rd) * 4) != cudaSuccess ||
       cudaMalloc(&h->rvt, vt_bytes) != cudaSuccess ||
       cudaMalloc(&h->status, 16) != cudaSuccess || cudaMemset(h->status, 0, 16) != cudaSuccess) {
     cudaGetLastError();
@@ -1580,6 +1586,8 @@ mot_status replay_args(mot_handle h, const void* q, const void* k, const void* v
   a.guide = guide;
   a.out = out;
   a.sel = h->rsel;
+  a.sel_stride = sel_row(d);
+  a.pad_first = 1;
   a.seq_lens = seq_lens;
   a.batch = batch;
   a.status = h->status;
@@ -1600,8 +1608,10 @@ mot_status mot_replay_select(mot_handle h, const void* guide, const int32_t* seq
   if (cudaSetDevice(h->device) != cudaSuccess) return MOT_ERR_CUDA;
   if (batch == 0) return MOT_OK;
   a.sel = sel;
+  a.sel_stride = h->rd.S;
+  a.pad_first = 0;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, st); }));
+  MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, h->num_sms, st); }));
   return MOT_OK;
 }
 
@@ -1634,17 +1644,12 @@ mot_status mot_replay_attention(mot_handle h, int32_t layer, const void* q, cons
                        [&] { return launch_replay_fmha(a, tmK, tmVt, st); }));
     return MOT_OK;
   }
-  if (!full && replay_gattn_supported(d)) {
-    // guided layer on the tensor cores: selection, then the gathered-row attention
-    MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, st); }));
-    MOT_CUDA_TRY(timed(h, "replay_attn_sparse", st,
-                       [&] { return launch_replay_gattn(a, h->num_sms, st); }));
-    return MOT_OK;
-  }
+  // guided layers attend to the gathered rows of the selection; so do the full layers that
+  // the tensor-core tiling does not take, over the rows 0..u
   if (!full)
-    MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, st); }));
+    MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, h->num_sms, st); }));
   MOT_CUDA_TRY(timed(h, full ? "replay_attn_full" : "replay_attn_sparse", st,
-                     [&] { return launch_replay_attn(a, st); }));
+                     [&] { return launch_replay_gather(a, h->num_sms, st); }));
   return MOT_OK;
 }
 

@@ -156,23 +156,6 @@ __device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr) {
   return d;
 }
 
-// Shared-memory matrix descriptor for an MN-major operand with 128-byte
-// swizzling: each 128-byte row holds 64 consecutive M (or N) elements of one
-// K index, 8 K rows form a 1024-byte atom (SBO = 1024 B to the next 8 K), and
-// the next 64 M elements start `lbo` bytes further (LBO).
-__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t saddr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>(1024u >> 4) << 32;
-  d |= static_cast<uint64_t>(1u) << 46;
-  d |= static_cast<uint64_t>(2u) << 61;
-  return d;
-}
-
-// Instruction-descriptor bit that marks A as MN-major ("transpose A").
-constexpr uint32_t kIdescAMajorMN = 1u << 15;
-
 // Instruction descriptor for kind::f16 with bf16 A/B, fp32 accumulator,
 // both operands K-major: D format (bits 4-5) = 1 (f32), A format (7-9) = 1
 // (bf16), B format (10-12) = 1 (bf16), N >> 3 (17-22), M >> 4 (24-28).
@@ -481,20 +464,6 @@ __device__ __forceinline__ void fence_proxy_async_cluster() {
 
 // True in exactly one lane of the (fully active) warp. Issuing tcgen05.mma
 // from a warp-uniform loop under elect.sync keeps its operands warp-uniform.
-// Warp-wide maximum of an fp32 value (every lane of the warp takes part).
-__device__ __forceinline__ float redux_max_f32(float v) {
-  float r;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-  return r;
-}
-
-// Warp-wide sum of an unsigned 32-bit value (every lane of the warp takes part).
-__device__ __forceinline__ uint32_t redux_add_u32(uint32_t v) {
-  uint32_t r;
-  asm volatile("redux.sync.add.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
-  return r;
-}
-
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
   asm volatile(

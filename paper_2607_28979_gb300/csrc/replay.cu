@@ -1,6 +1,5 @@
-// Replay attention of the post-translation phase (App. C.4) on sm_103a:
-// Top-S source-guided sparse attention, and full causal attention for the
-// L_Full bottom layers.
+// Replay attention of the post-translation phase (App. C.4) on sm_103a: the
+// Top-S selection of the source-guided layers, and V^T for the full layers.
 //
 //   replay_select_kernel  one warp per context row (b, u): the S positions j <= u
 //                         with the largest guidance score A[b][u][j] (ties to the
@@ -17,19 +16,9 @@
 //                         position. Rows past 4,096 positions take
 //   replay_select_stream_kernel, the same selection with the high and low byte as
 //                         the two digits, reading the row once per pass.
-//   replay_attn_kernel    one warp per (b, key/value head, u), no block barriers:
-//                         the query heads of the GQA group attend to the selected
-//                         rows (sparse) or to positions 0..u in 128-key chunks
-//                         with an online softmax (full). Each lane scores four keys
-//                         of the chunk against every query of the group (16-byte
-//                         key reads, the pre-scaled queries broadcast from the
-//                         warp's shared copy), the softmax runs on warp shuffles in
-//                         fp32, and each lane accumulates d / 32 output dimensions
-//                         over the chunk's value rows (the warp reads each row
-//                         once, coalesced).
 //   replay_vt_kernel      V -> V^T per layer for the full-attention kernel.
-//   The tensor-core kernels are in replay_fmha.cu (full causal attention) and
-//   replay_gattn.cu (guided attention).
+//   The attention kernels are in replay_fmha.cu (full causal attention on tcgen05) and
+//   replay_gather.cu (guided layers, and the full layers that tiling does not take).
 #include "replay_common.cuh"
 
 namespace mot {
@@ -87,6 +76,16 @@ __device__ __forceinline__ uint32_t ord16x2(uint32_t q) {
   return q ^ ((((q >> 15) & 0x00010001u) * 0xFFFFu) | 0x80008000u);
 }
 
+// A full row of S entries in a workspace of wider rows: the rest repeats its first position.
+__device__ __forceinline__ void pad_row(const ReplayArgs& a, int32_t* out) {
+  const int lane = threadIdx.x & 31;
+  if (a.sel_stride > a.d.S) {
+    __syncwarp();
+    const int32_t first = *static_cast<volatile int32_t*>(out);
+    for (int j = a.d.S + lane; j < a.sel_stride; j += 32) out[j] = first;
+  }
+}
+
 // Selection for any max_seq. One warp per context row (b, u). With o = the
 // order-preserving 16 bits of a score, the S-th largest (o, -j) key is found in
 // two histogram passes over o (high byte, then low byte): V = its score bits, k =
@@ -102,10 +101,10 @@ __global__ void __launch_bounds__(32 * kSelWarps) replay_select_stream_kernel(co
   if (row >= d.B * d.N) return;
   const int b = row / d.N, u = row - b * d.N;
   if (u >= seq_len_of(a, b)) return;
-  int32_t* out = a.sel + int64_t(row) * d.S;
+  int32_t* out = a.sel + int64_t(row) * a.sel_stride;
   const int n = u + 1;
   if (n <= d.S) {
-    for (int j = lane; j < d.S; j += 32) out[j] = j < n ? j : -1;
+    for (int j = lane; j < a.sel_stride; j += 32) out[j] = j < n ? j : a.pad_first ? 0 : -1;
     return;
   }
   const uint16_t* A = static_cast<const uint16_t*>(a.guide) + int64_t(row) * d.N;
@@ -181,6 +180,7 @@ __global__ void __launch_bounds__(32 * kSelWarps) replay_select_stream_kernel(co
     base += sel_tot;
     eq_taken += eq_tot;
   }
+  pad_row(a, out);
 }
 
 // Selection for max_seq <= 4096, with the row's keys cached in shared memory.
@@ -208,10 +208,10 @@ __global__ void __launch_bounds__(32 * kSelCacheWarps) replay_select_kernel(cons
   if (row >= d.B * d.N) return;
   const int b = row / d.N, u = row - b * d.N;
   if (u >= seq_len_of(a, b)) return;
-  int32_t* out = a.sel + int64_t(row) * d.S;
+  int32_t* out = a.sel + int64_t(row) * a.sel_stride;
   const int n = u + 1;
   if (n <= d.S) {
-    for (int j = lane; j < d.S; j += 32) out[j] = j < n ? j : -1;
+    for (int j = lane; j < a.sel_stride; j += 32) out[j] = j < n ? j : a.pad_first ? 0 : -1;
     return;
   }
   const uint16_t* A = static_cast<const uint16_t*>(a.guide) + int64_t(row) * d.N;
@@ -365,165 +365,7 @@ __global__ void __launch_bounds__(32 * kSelCacheWarps) replay_select_kernel(cons
     for (uint32_t m = sel; m != 0u; m &= m - 1u) out[pos++] = j8 + __ffs(m) - 1;
     base += sel_tot;
   }
-}
-
-constexpr int kAttnWarps = 4;   // (b, key/value head, u) items per CTA, one warp each
-
-// Shared memory of one warp: the group's pre-scaled queries [G][D], the chunk's
-// probabilities [G][128] and its key positions [128].
-template <int D, int G>
-__host__ __device__ constexpr int attn_warp_floats() { return G * D + G * 128 + 128; }
-
-// Residency floor per group size: the gathers are latency-bound, so small groups
-// trade a few spilled registers for more resident warps.
-__host__ __device__ constexpr int attn_min_blocks(int g) { return g <= 8 ? 4 : 1; }
-
-template <int D, int G>
-__global__ void __launch_bounds__(32 * kAttnWarps, attn_min_blocks(G))
-    replay_attn_kernel(const ReplayArgs a) {
-  constexpr int DL = D / 32;   // output dimensions per lane
-  extern __shared__ float4 attn_smem4[];
-  const ReplayDims& d = a.d;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t item = int64_t(blockIdx.x) * kAttnWarps + warp;
-  if (item >= int64_t(d.B) * d.Hkv * d.N) return;
-  const int u = static_cast<int>(item % d.N);
-  const int bh = static_cast<int>(item / d.N);
-  const int hk = bh % d.Hkv, b = bh / d.Hkv;
-  if (u >= seq_len_of(a, b)) return;
-  float* ws = reinterpret_cast<float*>(attn_smem4) + warp * attn_warp_floats<D, G>();
-  float* qs = ws;                        // [G][D]
-  float* ps = ws + G * D;                // [G][128]
-  int32_t* ix = reinterpret_cast<int32_t*>(ps + G * 128);   // [128]
-  const float scale = rsqrtf(float(D));
-  for (int i = lane; i < G * D; i += 32) {
-    const int g = i / D, c = i - g * D;
-    qs[i] = bf16f(static_cast<const uint16_t*>(a.q)[((int64_t(b) * d.Hq + hk * G + g) * d.N + u) * D + c]) *
-            scale;
-  }
-  const bool full = a.full != 0;
-  const int n_keys = full ? u + 1 : min(d.S, u + 1);
-  const int32_t* sel = a.sel + (int64_t(b) * d.N + u) * d.S;
-  const uint16_t* kb = static_cast<const uint16_t*>(a.k) + (int64_t(b) * d.Hkv + hk) * d.N * D;
-  const uint16_t* vb = static_cast<const uint16_t*>(a.v) + (int64_t(b) * d.Hkv + hk) * d.N * D;
-  float m[G], l[G], acc[G][DL];
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    m[g] = -INFINITY;
-    l[g] = 0.f;
-#pragma unroll
-    for (int e = 0; e < DL; ++e) acc[g][e] = 0.f;
-  }
-  __syncwarp();
-  for (int c0 = 0; c0 < n_keys; c0 += 128) {
-    const int nc = min(128, n_keys - c0);
-    // this lane's keys: chunk positions lane, lane + 32, lane + 64, lane + 96
-    int j[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int t = lane + 32 * i;
-      j[i] = t < nc ? (full ? c0 + t : sel[c0 + t]) : -1;
-      ix[t] = j[i];
-    }
-    float s[4][G];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int g = 0; g < G; ++g) s[i][g] = 0.f;
-#pragma unroll 2
-    for (int c = 0; c < D / 8; ++c) {
-      float kf[4][8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (j[i] >= 0) w = __ldg(reinterpret_cast<const uint4*>(kb + int64_t(j[i]) * D) + c);
-        kf[i][0] = __uint_as_float(w.x << 16); kf[i][1] = __uint_as_float(w.x & 0xFFFF0000u);
-        kf[i][2] = __uint_as_float(w.y << 16); kf[i][3] = __uint_as_float(w.y & 0xFFFF0000u);
-        kf[i][4] = __uint_as_float(w.z << 16); kf[i][5] = __uint_as_float(w.z & 0xFFFF0000u);
-        kf[i][6] = __uint_as_float(w.w << 16); kf[i][7] = __uint_as_float(w.w & 0xFFFF0000u);
-      }
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const float4 q0 = *reinterpret_cast<const float4*>(qs + g * D + 8 * c);
-        const float4 q1 = *reinterpret_cast<const float4*>(qs + g * D + 8 * c + 4);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float x = s[i][g];
-          x = fmaf(q0.x, kf[i][0], x); x = fmaf(q0.y, kf[i][1], x);
-          x = fmaf(q0.z, kf[i][2], x); x = fmaf(q0.w, kf[i][3], x);
-          x = fmaf(q1.x, kf[i][4], x); x = fmaf(q1.y, kf[i][5], x);
-          x = fmaf(q1.z, kf[i][6], x); x = fmaf(q1.w, kf[i][7], x);
-          s[i][g] = x;
-        }
-      }
-    }
-    // online softmax per query of the group (warp reductions only)
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float mx = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (j[i] >= 0) mx = fmaxf(mx, s[i][g]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float mnew = fmaxf(m[g], mx);
-      const float corr = m[g] == -INFINITY ? 0.f : expf(m[g] - mnew);
-      float sum = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float pv = j[i] >= 0 ? expf(s[i][g] - mnew) : 0.f;
-        ps[g * 128 + lane + 32 * i] = pv;
-        sum += pv;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      l[g] = l[g] * corr + sum;
-      m[g] = mnew;
-#pragma unroll
-      for (int e = 0; e < DL; ++e) acc[g][e] *= corr;
-    }
-    __syncwarp();
-    // weighted value rows: this lane's DL dimensions of every selected row
-    for (int t0 = 0; t0 < nc; t0 += 4) {
-      float pq[G][4];
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const float4 p4 = *reinterpret_cast<const float4*>(ps + g * 128 + t0);
-        pq[g][0] = p4.x; pq[g][1] = p4.y; pq[g][2] = p4.z; pq[g][3] = p4.w;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (t0 + i >= nc) break;
-        const uint16_t* vr = vb + int64_t(ix[t0 + i]) * D + lane * DL;
-        float vv[DL];
-        if constexpr (DL == 4) {
-          const uint2 w = __ldg(reinterpret_cast<const uint2*>(vr));
-          vv[0] = __uint_as_float(w.x << 16); vv[1] = __uint_as_float(w.x & 0xFFFF0000u);
-          vv[2] = __uint_as_float(w.y << 16); vv[3] = __uint_as_float(w.y & 0xFFFF0000u);
-        } else {
-          const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(vr));
-          vv[0] = __uint_as_float(w << 16); vv[1] = __uint_as_float(w & 0xFFFF0000u);
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g)
-#pragma unroll
-          for (int e = 0; e < DL; ++e) acc[g][e] = fmaf(pq[g][i], vv[e], acc[g][e]);
-      }
-    }
-    __syncwarp();
-  }
-  uint16_t* o = static_cast<uint16_t*>(a.out);
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const float inv = 1.f / l[g];
-    uint16_t* orow = o + ((int64_t(b) * d.Hq + hk * G + g) * d.N + u) * D + lane * DL;
-    if constexpr (DL == 4) {
-      *reinterpret_cast<uint2*>(orow) = make_uint2(pack_bf16(acc[g][0] * inv, acc[g][1] * inv),
-                                                   pack_bf16(acc[g][2] * inv, acc[g][3] * inv));
-    } else {
-      *reinterpret_cast<uint32_t*>(orow) = pack_bf16(acc[g][0] * inv, acc[g][1] * inv);
-    }
-  }
+  pad_row(a, out);
 }
 
 // ---------------------------------------------------------------- V^T for the tensor-core path
@@ -554,7 +396,7 @@ bool replay_supported(const ReplayDims& d) {
          (d.d == 64 || d.d == 128) && d.S >= 1 && d.S <= 4096 && d.N >= 1 && d.N <= 65536;
 }
 
-cudaError_t launch_replay_select(const ReplayArgs& a, cudaStream_t st) {
+cudaError_t launch_replay_select(const ReplayArgs& a, int, cudaStream_t st) {
   const int rows = a.d.B * a.d.N;
   if (rows <= 0) return cudaSuccess;
   if (a.d.N <= 256 * kSelCacheRounds)
@@ -570,34 +412,5 @@ cudaError_t launch_replay_vt(const ReplayArgs& a, void* vt, cudaStream_t st) {
   replay_vt_kernel<<<grid, 256, 0, st>>>(static_cast<const uint16_t*>(a.v),
                                          static_cast<uint16_t*>(vt), d.N, d.d);
   return cudaGetLastError();
-}
-
-template <int D, int G>
-cudaError_t launch_attn_dg(const ReplayArgs& a, cudaStream_t st) {
-  const size_t smem = size_t(kAttnWarps) * attn_warp_floats<D, G>() * 4;
-  static bool attr = false;
-  if (!attr && smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(replay_attn_kernel<D, G>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-  }
-  attr = true;
-  const int64_t items = int64_t(a.d.B) * a.d.Hkv * a.d.N;
-  const unsigned grid = static_cast<unsigned>((items + kAttnWarps - 1) / kAttnWarps);
-  replay_attn_kernel<D, G><<<grid, 32 * kAttnWarps, smem, st>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_replay_attn(const ReplayArgs& a, cudaStream_t st) {
-  const int G = a.d.Hq / a.d.Hkv;
-#define MOT_RP_CASE(GG)                                                             \
-  case GG:                                                                          \
-    return a.d.d == 128 ? launch_attn_dg<128, GG>(a, st) : launch_attn_dg<64, GG>(a, st);
-  switch (G) {
-    MOT_RP_CASE(1) MOT_RP_CASE(2) MOT_RP_CASE(3) MOT_RP_CASE(4) MOT_RP_CASE(5)
-    MOT_RP_CASE(6) MOT_RP_CASE(7) MOT_RP_CASE(8) MOT_RP_CASE(12) MOT_RP_CASE(16)
-    default: return cudaErrorInvalidValue;
-  }
-#undef MOT_RP_CASE
 }
 }  // namespace mot

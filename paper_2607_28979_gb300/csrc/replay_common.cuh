@@ -1,6 +1,6 @@
 // Helpers shared by the replay attention kernels (App. C.4): replay.cu (selection,
-// SIMT attention, V transpose), replay_fmha.cu (full causal attention on the tensor
-// cores) and replay_gattn.cu (source-guided attention on the tensor cores).
+// V transpose), replay_fmha.cu (full causal attention on tcgen05) and replay_gather.cu
+// (attention over gathered rows).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -10,7 +10,7 @@
 
 namespace mot {
 
-// GQA group sizes with an instantiated attention kernel
+// GQA group sizes the attention takes
 __host__ __device__ constexpr bool group_ok(int g) {
   return (g >= 1 && g <= 8) || g == 12 || g == 16;
 }

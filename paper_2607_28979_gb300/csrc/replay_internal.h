@@ -1,5 +1,5 @@
 // Internal declarations of the replay attention (replay.cu, replay_fmha.cu,
-// replay_gattn.cu), shared with the C-ABI layer.
+// replay_gather.cu), shared with the C-ABI layer.
 #pragma once
 
 #include "mot_internal.h"
@@ -24,12 +24,14 @@ struct ReplayArgs {
   const void* guide;
   void* out;
   int32_t* sel;
+  int64_t sel_stride;     // entries from one row of sel to the next
+  int32_t pad_first;      // fill a row's unused entries with its first position (else -1)
   const int32_t* seq_lens;
   int32_t batch;
   int32_t full;   // 1: attend to every position 0..u
   int32_t* status;
   long long wait_limit;   // bound of every pipeline wait (SM cycles)
-  int32_t stall_test;     // test hook: the guided kernel's first CTA stalls its first MMA barrier
+  int32_t stall_test;     // test hook: the gather kernel's first CTA waits for a signal nothing sends
 };
 bool replay_supported(const ReplayDims& d);
 // Full causal attention on the tensor cores: maps over k [B*Hkv*N][d] (box
@@ -39,11 +41,11 @@ bool replay_fmha_supported(const ReplayDims& d);
 cudaError_t launch_replay_vt(const ReplayArgs& a, void* vt, cudaStream_t st);
 cudaError_t launch_replay_fmha(const ReplayArgs& a, const CUtensorMap& tmK,
                                const CUtensorMap& tmVt, cudaStream_t st);
-cudaError_t launch_replay_select(const ReplayArgs& a, cudaStream_t st);
-// Guided layers on the tensor cores (d = 128, GQA groups of up to 16, S <= 128):
-// persistent CTAs, as many per SM as fit.
-bool replay_gattn_supported(const ReplayDims& d);
-cudaError_t launch_replay_gattn(const ReplayArgs& a, int num_sms, cudaStream_t st);
-cudaError_t launch_replay_attn(const ReplayArgs& a, cudaStream_t st);
+cudaError_t launch_replay_select(const ReplayArgs& a, int num_sms, cudaStream_t st);
+// Guided layers, and full layers that launch_replay_fmha does not take. The rows of a.sel are
+// whole units of replay_gather_unit(d) entries, the unused ones filled (pad_first) with a
+// position of the set. Persistent, one CTA per SM.
+int replay_gather_unit(const ReplayDims& d);
+cudaError_t launch_replay_gather(const ReplayArgs& a, int num_sms, cudaStream_t st);
 
 }  // namespace mot

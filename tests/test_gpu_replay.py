@@ -304,3 +304,34 @@ def test_guided_timeout_is_reported_and_recovers():
                 tb.append(b); th.append(h); tu.append(u)
     ref = oracle.replay_tokens(wl, layer, q, k, v, g, tb, th, tu)
     G.assert_parity(BF16, _f64(out)[tb, th, tu], ref, "guided layer after a timeout")
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("group,top_s,n", [(1, 1, 70), (4, 31, 130), (5, 32, 131), (8, 33, 99), (6, 64, 201),
+                                           (3, 65, 200), (16, 127, 260), (2, 129, 333), (7, 192, 257),
+                                           (12, 200, 333)])
+def test_gathered_rows_every_unit_size(d, group, top_s, n):
+    """The gather kernel at the edges of its units (32, 64 or 128 rows, 64 for larger sets),
+    in every form of the probabilities (group sizes up to 4, 8 and 16), with a context that
+    is not a multiple of 8 so that the full layer takes it too. Against the oracle, with
+    the parity bar of the other replay tests."""
+    wl = RW(f"r_u{top_s}", 2, 3, group * 2, 2, d, 2, n, (n, n // 2 + 1), top_s=top_s, n_full=1)
+    if n % 8 == 0:
+        wl = wl.replace(max_seq=n + 1)
+    q, k, v = synth.gen_replay_qkv(wl, 37)
+    g = synth.gen_guide(wl, 41)
+    run = ReplayRun(wl)
+    rng = np.random.default_rng(top_s)
+    for layer in (0, 2):
+        out = run.attend(layer, q, k, v, None if layer < wl.n_full else g)
+        tb, th, tu = [], [], []
+        for b, L in enumerate(wl.seq_lens):
+            edge = [x for x in (0, 15, 16, 63, 64, top_s - 1, top_s, L - 1) if x < L]
+            for u in np.unique(np.concatenate([edge, rng.integers(0, L, size=8)])):
+                for h in range(wl.q_heads):
+                    tb.append(b); th.append(h); tu.append(int(u))
+        ref = oracle.replay_tokens(wl, layer, q, k, v, g, tb, th, tu)
+        G.assert_parity(BF16, _f64(out)[tb, th, tu], ref, f"d {d} group {group} S {top_s} layer {layer}")
+        o = out.cpu().numpy()
+        for b, L in enumerate(wl.seq_lens):
+            assert (o[b, :, L:] == np.int16(G.SENTINEL_BF16)).all()
