@@ -335,3 +335,34 @@ def test_gathered_rows_every_unit_size(d, group, top_s, n):
         o = out.cpu().numpy()
         for b, L in enumerate(wl.seq_lens):
             assert (o[b, :, L:] == np.int16(G.SENTINEL_BF16)).all()
+
+
+@pytest.mark.parametrize("max_seq", [257, 263, 520, 1030, 2049, 4093])   # every 16-byte phase of a row start
+@pytest.mark.parametrize("top_s", [1, 128, 160, 161, 256, 449])
+def test_selection_bounds_lists_and_fallback(max_seq, top_s):
+    """The bounded selection against numpy, bit for bit: one or two sets of group maxima
+    (top_s up to 160 and 448) and the histogram past them; rows whose candidates overflow
+    the list (a few values only), rows of distinct scores, mixed signs, and rows holding the
+    lowest key (a negative NaN pattern), whose bound cannot separate it from empty slots."""
+    wl = RW("r_bound", 2, 2, 1, 1, 64, 2, max_seq, (max_seq, max_seq - 3), top_s=top_s, n_full=1)
+    rng = np.random.default_rng(max_seq * 1000 + top_s)
+    N = max_seq
+    g = rng.integers(0x0080, 0x7F00, size=(2, N, N)).astype(np.uint16)
+    g[0, 1::6] = rng.integers(0x3F80, 0x3F84, size=g[0, 1::6].shape).astype(np.uint16)
+    g[0, 2::6] = (np.exp(rng.standard_normal(g[0, 2::6].shape)).astype(np.float32).view(np.uint32) >> 16)
+    g[0, 3::6] = (rng.standard_normal(g[0, 3::6].shape).astype(np.float32).view(np.uint32) >> 16)
+    g[0, 4::6] = np.where(rng.random(g[0, 4::6].shape) < 0.9, 0xFFFF, 0x3F80)
+    g[0, 5::6] = np.where(rng.random(g[0, 5::6].shape) < 0.5, 0, 0x3F80)
+    g[1, 1::3] = rng.integers(0, 0x0100, size=g[1, 1::3].shape)      # subnormals
+    g[1, 2::3, 5::64] = rng.choice([0x7F80, 0x7FC0, 0x8000], size=g[1, 2::3, 5::64].shape)
+    sel = ReplayRun(wl).select(g)
+    for b, L in enumerate(wl.seq_lens):
+        for u in np.unique(np.concatenate([[0, top_s - 1, top_s, 255, 256, L - 1],
+                                           rng.integers(0, L, size=60)])):
+            if u >= L:
+                continue
+            bits = g[b, u, :u + 1].astype(np.int64)
+            key = np.where(bits >= 0x8000, 0xFFFF - bits, bits | 0x8000)
+            ref = np.sort(np.lexsort((np.arange(u + 1), -key))[:top_s])
+            np.testing.assert_array_equal(sel[b, u, :ref.size], ref, err_msg=f"b={b} u={u}")
+            assert (sel[b, u, ref.size:] == -1).all()
