@@ -176,7 +176,8 @@ KERNEL_SOURCES = {
     "replay_fmha_full": ["replay_fmha.cu", "replay_common.cuh", "replay_internal.h",
                          "mot_internal.h", "ptx.cuh"],
     # backbone translators (all kernels of bt.cu)
-    "bt_ffn_fused": ["bt.cu", "bt_internal.h", "gelu.cuh", "mot_internal.h", "ptx.cuh"],
+    "bt_ffn_fused": ["bt.cu", "bt_common.cuh", "bt_internal.h", "gelu.cuh", "mot_internal.h",
+                     "ptx.cuh"],
 }
 
 

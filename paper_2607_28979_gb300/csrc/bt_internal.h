@@ -62,6 +62,8 @@ struct BtArgs {
   void* f;               // bf16 FFN hidden                    [df]
   void* xo;              // bf16 h_r (raw)                     [d] (= [B * S][P * d])
   float2* rstat;         // [G][R] (mean, M2) of each h_r row over its d values
+  int32_t xo_tok0;       // token rows before this slot's in xo (the scan keeps one block per slot)
+  const float* prm;      // [G][N][bt_scan_prm_floats] the scan's fp32 vectors of each slot
   int32_t* status;
   long long wait_limit;
   // Top-1 routing (token buckets): group g's row space holds only the tokens
@@ -103,5 +105,18 @@ cudaError_t launch_bt_gemm(int mode, const BtArgs& a, const CUtensorMap& tmA,
 // map with box 64 x 128, W_F2 map with box 64 x d; ends with kBtF2's row epilogue.
 cudaError_t launch_bt_ffn(const BtArgs& a, const CUtensorMap& tmXf, const CUtensorMap& tmW1,
                           const CUtensorMap& tmW2, int num_sms, cudaStream_t st);
+
+
+// The whole scan in one launch (bt_scan.cu): h_r rows and their statistics of every slot into
+// xo [N][G][R][d] and rstat [N][G][R]. tm: W_in, W_Q, W_K|V, W_O, W_F1 and W_F2, all as boxes
+// of 128 rows x 64. Routed, the source rows are gathered through the bucket lists.
+struct BtScanVecs {      // host arrays at load: s_in, c_in [G][..], the others [G][N][..]
+  const float *s_in, *c_in, *ln_c, *ln_q, *ln_f, *c_q, *c_kv, *c_o, *c_f1, *c_f2;
+};
+bool bt_scan_supported(const BtDims& d);
+int bt_scan_prm_floats(const BtDims& d);
+void bt_scan_pack_prm(const BtDims& d, const BtScanVecs& v, int g, int slot, float* out);
+cudaError_t launch_bt_scan(const BtArgs& a, const CUtensorMap (&tm)[6], int num_sms,
+                           cudaStream_t st);
 
 }  // namespace mot

@@ -96,6 +96,10 @@ struct BtState {
   // Top-1 routing (token buckets): counts, lists, tile prefixes, packed source rows
   int32_t *rcnt = nullptr, *rlist = nullptr, *rpre = nullptr;
   void* xs = nullptr;   // [G][R][d_s] bf16
+  // the scan in one launch: xo and rstat then hold every slot, and the hidden rows f nothing
+  bool scan = false;
+  float* prm = nullptr;   // [G][N] fp32 vectors of the scan
+  CUtensorMap tm_wkvh{};
   CUtensorMap tm_win{}, tm_wq{}, tm_wkv{}, tm_wo{}, tm_wf1{}, tm_wf2{}, tm_wout{}, tm_wf1c{};
   CUtensorMap tm_xz{}, tm_xq{}, tm_o{}, tm_xf{}, tm_f{}, tm_xo{};
   CUtensorMap tm_xs{}, tm_wout_r{};   // routed: packed source rows, W_out with 256-row boxes
@@ -103,7 +107,7 @@ struct BtState {
   void free_all() {
     void* ptrs[] = {wg, bg, s_in, c_in, c_q, c_kv, c_o, c_f1, c_f2, c_out, s_out, ln_q, ln_c,
                     ln_f, win, wq, wkv, wo, wf1, wf2, wout, gate, h, ht, xz, xq, q, kv, o, xf,
-                    f, xo, rstat, rcnt, rlist, rpre, xs};
+                    f, xo, rstat, rcnt, rlist, rpre, xs, prm};
     for (void* p : ptrs)
       if (p) cudaFree(p);
   }
@@ -860,13 +864,16 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
   h->use_umma = true;
 
   const size_t G = bd.G, N = bd.N, D = bd.d, df = bd.df, R = size_t(bd.R), E = bd.E;
+  bt.scan = bt_scan_supported(bd) && int64_t(N) * bd.G * bd.B * bd.S <= INT32_MAX / 2;
+  const size_t slots = bt.scan ? N : 1;
   struct A { void** p; size_t n; } allocs[] = {
+      {(void**)&bt.prm, bt.scan ? G * N * bt_scan_prm_floats(bd) * 4 : 16},
       {&bt.wg, 2 * E * N * bd.Ds * 2}, {(void**)&bt.bg, 2 * E * 4},
       {(void**)&bt.s_in, G * D * 4}, {(void**)&bt.c_in, G * D * 4},
       {(void**)&bt.c_q, G * N * D * 4}, {(void**)&bt.c_kv, G * N * 2 * D * 4},
       {(void**)&bt.c_o, G * N * D * 4}, {(void**)&bt.c_f1, G * N * df * 4},
       {(void**)&bt.c_f2, G * N * D * 4}, {(void**)&bt.c_out, G * bd.Dt * 4},
-      {(void**)&bt.s_out, G * bd.Dt * 4}, {(void**)&bt.rstat, G * R * 8},
+      {(void**)&bt.s_out, G * bd.Dt * 4}, {(void**)&bt.rstat, slots * G * R * 8},
       {(void**)&bt.ln_q, G * N * 2 * D * 4}, {(void**)&bt.ln_c, G * N * 2 * D * 4},
       {(void**)&bt.ln_f, G * N * 2 * D * 4},
       {&bt.win, G * D * 2 * bd.d_s * 2}, {&bt.wq, G * N * D * D * 2}, {&bt.wkv, G * N * 2 * D * D * 2},
@@ -876,7 +883,7 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
       {(void**)&bt.h, G * R * D * 4}, {(void**)&bt.ht, G * R * D * 4},
       {&bt.xz, G * R * D * 2}, {&bt.xq, G * R * D * 2}, {&bt.q, G * R * D * 2},
       {&bt.kv, G * R * 2 * D * 2}, {&bt.o, G * R * D * 2}, {&bt.xf, G * R * D * 2},
-      {&bt.f, G * R * df * 2}, {&bt.xo, G * R * D * 2},
+      {&bt.f, df % 128 ? G * R * df * 2 : 16}, {&bt.xo, slots * G * R * D * 2},
       {(void**)&bt.rcnt, 64 * 4}, {(void**)&bt.rlist, G * size_t(bd.B) * bd.S * 4},
       {(void**)&bt.rpre, (2 * G + 2) * 4},
       {&bt.xs, bd.top_k == 1 ? G * R * bd.d_s * 2 : 16},
@@ -910,6 +917,7 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
   map2(&bt.tm_win, bt.win, 2 * bd.d_s, G * D, uint32_t(D));
   map2(&bt.tm_wq, bt.wq, D, G * N * D, uint32_t(D));
   map2(&bt.tm_wkv, bt.wkv, D, G * N * 2 * D, uint32_t(2 * D));
+  map2(&bt.tm_wkvh, bt.wkv, D, G * N * 2 * D, uint32_t(D));
   map2(&bt.tm_wo, bt.wo, D, G * N * D, uint32_t(D));
   map2(&bt.tm_wf1, bt.wf1, D, G * N * df, nt_f1);
   map2(&bt.tm_wf1c, bt.wf1, D, G * N * df, 128);   // 128-row chunks for the fused FFN
@@ -920,8 +928,8 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
   map2(&bt.tm_xq, bt.xq, D, G * R, 128);
   map2(&bt.tm_o, bt.o, D, G * R, 128);
   map2(&bt.tm_xf, bt.xf, D, G * R, 128);
-  map2(&bt.tm_f, bt.f, df, G * R, 128);
-  map2(&bt.tm_xo, bt.xo, uint64_t(bd.P) * D, G * size_t(bd.B) * bd.S, 128);
+  if (df % 128) map2(&bt.tm_f, bt.f, df, G * R, 128);
+  map2(&bt.tm_xo, bt.xo, uint64_t(bd.P) * D, slots * G * size_t(bd.B) * bd.S, 128);
   if (bd.top_k == 1) {   // Top-1 routing (the default for these handles): token buckets
     uint32_t nt_r = 256;
     while (nt_r > 32 && bd.Dt % nt_r) nt_r -= 32;
@@ -1031,7 +1039,18 @@ mot_status bt_load(mot_ctx* h, const void* host_blob, size_t bytes) {
     }
     if (off != (x + 1) * blk) return MOT_ERR_WEIGHTS_SIZE;   // layout bookkeeping check
   }
+  std::vector<float> prm;
+  if (bt.scan) {
+    const size_t n = bt_scan_prm_floats(d);
+    prm.resize(G * N * n);
+    const BtScanVecs v{s_in.data(), c_in.data(), ln_c.data(), ln_q.data(), ln_f.data(),
+                       c_q.data(),  c_kv.data(), c_o.data(),  c_f1.data(), c_f2.data()};
+    for (size_t g = 0; g < G; ++g)
+      for (size_t r = 0; r < N; ++r)
+        bt_scan_pack_prm(d, v, int(g), int(r), &prm[(g * N + r) * n]);
+  }
   struct U { void* dst; const void* src; size_t n; } ups[] = {
+      {bt.prm, prm.data(), prm.size() * 4},
       {bt.wg, wg.data(), wg.size() * 2}, {bt.bg, bg.data(), bg.size() * 4},
       {bt.win, win.data(), win.size() * 2}, {bt.s_in, s_in.data(), s_in.size() * 4},
       {bt.c_in, c_in.data(), c_in.size() * 4}, {bt.wq, wq.data(), wq.size() * 2},
@@ -1481,6 +1500,25 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
       return launch_bt_route(a, bt.rcnt, bt.rlist, bt.rpre, st);
     }));
   }
+  auto project = [&](int r) {   // the output projection of slot r
+    a.slot = r;
+    return timed(h, "bt_out_gelu_combine", st, [&] {
+      return launch_bt_gemm(kBtOut, a, bt.tm_xo, bt.tm_xo, routed ? bt.tm_wout_r : bt.tm_wout,
+                            h->num_sms, st);
+    });
+  };
+  if (bt.scan && !h->profile) {   // profiling times the stages one by one
+    a.prm = bt.prm;
+    const CUtensorMap tm[6] = {bt.tm_win, bt.tm_wq, bt.tm_wkvh, bt.tm_wo, bt.tm_wf1c, bt.tm_wf2};
+    MOT_CUDA_TRY(timed(h, "bt_scan", st, [&] { return launch_bt_scan(a, tm, h->num_sms, st); }));
+    for (int r = 0; r < d.N; ++r) {
+      a.xo_tok0 = r * d.G * d.B * d.S;
+      a.rstat = bt.rstat + size_t(r) * d.G * d.R;
+      MOT_CUDA_TRY(project(r));
+    }
+    if (routed) h->counts_valid = true;
+    return MOT_OK;
+  }
   for (int r = 0; r < d.N; ++r) {
     a.slot = r;
     if (routed)
@@ -1511,10 +1549,7 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
         return launch_bt_gemm(kBtF2, a, bt.tm_f, bt.tm_f, bt.tm_wf2, h->num_sms, st);
       }));
     }
-    MOT_CUDA_TRY(timed(h, "bt_out_gelu_combine", st, [&] {
-      return launch_bt_gemm(kBtOut, a, bt.tm_xo, bt.tm_xo, routed ? bt.tm_wout_r : bt.tm_wout,
-                            h->num_sms, st);
-    }));
+    MOT_CUDA_TRY(project(r));
   }
   if (routed) h->counts_valid = true;
   return MOT_OK;

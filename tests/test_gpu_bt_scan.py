@@ -1,0 +1,104 @@
+"""The backbone translators' scan in one launch, at the edges of its tiles, chunks and
+attention blocks: against the fp64 oracle, and against the staged schedule (which runs
+while profiling is enabled) for what must agree bit for bit or position by position."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import _gpu as G   # noqa: E402
+M = G.M
+
+W = synth.Workload
+# name: (source heads P, d_s, target heads, d_t, E, top_k, lengths, (window start, slots, 128, heads, d_f))
+SHAPES = {
+    "p5_ds128_dh16": (5, 128, 3, 32, 1, 0, (26, 25, 1), (0, 2, 128, 8, 128)),    # one FFN chunk, 3-token blocks
+    "p16_dh64": (16, 64, 2, 64, 2, 1, (8, 9, 17), (1, 3, 128, 2, 256)),           # whole 16-row blocks, two chunks
+    "p7_dh32": (7, 64, 4, 32, 3, 0, (18, 19, 37), (0, 2, 128, 4, 768)),           # 126 rows, six chunks
+    "p1_dh16": (1, 128, 2, 32, 2, 0, (127, 128, 129), (2, 1, 128, 8, 512)),       # 16-token blocks, one slot
+    "p9_top1": (9, 64, 2, 128, 4, 1, (14, 15, 0, 29), (0, 4, 128, 4, 1024)),      # 9 of 16 rows, shorter ring
+}
+
+
+def _run(wl, sk, sv, blob, staged=False):
+    h = M.mot_create_bt(*M.bt_config_from(wl))
+    M.mot_load_weights(h, blob)
+    M.mot_profile_enable(h, staged)
+    k, v = G.to_device(wl, sk), G.to_device(wl, sv)
+    (bk, dk), (bv, dv) = G.alloc_dst(wl), G.alloc_dst(wl)
+    lens = torch.tensor(wl.seq_lens, dtype=torch.int32, device="cuda")
+    c0 = M.mot_get_launch_count(h)
+    M.mot_translate_bt(h, k, v, lens, wl.batch, dk, dv)
+    assert M.mot_get_device_status(h) == M.MOT_OK
+    return dk, dv, M.mot_get_launch_count(h) - c0
+
+
+def _workload(name):
+    P, ds, ht, dt, e, top_k, lens, bt = SHAPES[name]
+    return W(name, 3, P, ds, 5, ht, dt, e, 0, len(lens), max(lens), "bf16", lens, top_k=top_k, bt=bt)
+
+
+def _inputs(wl, seed):
+    return synth.gen_cache(wl, 0, seed), synth.gen_cache(wl, 1, seed), synth.gen_weights(wl, seed)
+
+
+@pytest.mark.parametrize("name", sorted(SHAPES))
+def test_scan_matches_oracle(name):
+    wl = _workload(name)
+    sk, sv, blob = _inputs(wl, 5)
+    dk, dv, launches = _run(wl, sk, sv, blob)
+    sdk, sdv, staged = _run(wl, sk, sv, blob, staged=True)
+    assert launches < staged
+    tb, ts = zip(*[(b, s) for b, n in enumerate(wl.seq_lens) for s in range(n)])
+    tb, ts = np.array(tb), np.array(ts)
+    ref = oracle.bt_tokens(wl, sk, sv, blob, tb, ts)
+    if 0 < wl.top_k < wl.n_translators:   # tokens whose two best scores nearly tie may go either way
+        g = oracle.bt_tokens(wl.replace(top_k=0), sk, sv, blob, tb, ts, want_gate=True)[1]
+        top = np.sort(g, axis=2)
+        clear = top[:, :, -1] - top[:, :, -2] > 1e-4
+    else:
+        clear = np.ones((2, tb.size), dtype=bool)
+    win = set(wl.bt_window)
+    for X, (dst, other) in enumerate(((dk, sdk), (dv, sdv))):
+        got = dst.double().cpu().numpy()
+        for r, l in enumerate(wl.bt_window):
+            rows = got[l][tb, :, ts].reshape(tb.size, -1)
+            G.assert_parity(wl, rows[clear[X]], ref[r][X][clear[X]], f"{name} X={X} slot {r}")
+        # what is written is exactly what the staged schedule writes
+        s = G.sentinel_value(wl)
+        assert torch.equal(G.int_view(dst) == s, G.int_view(other) == s)
+        for l in range(wl.n_layers_tgt):
+            if l not in win:
+                assert bool((G.int_view(dst)[l] == s).all())
+
+
+def test_scan_keeps_non_finite_tokens_apart():
+    """A NaN or infinity in one token's rows makes that token's outputs NaN and leaves every
+    other token as it was, also those that share its attention blocks."""
+    wl = _workload("p5_ds128_dh16")
+    sk, sv, blob = _inputs(wl, 7)
+    clean = _run(wl, sk, sv, blob)
+    bad = [(0, 3, 0x7FC0), (0, 4, 0x7F80), (1, 24, 0xFF80), (2, 0, 0x7FC0)]
+    sk2, sv2 = sk.copy(), sv.copy()
+    for b, s, bits in bad:
+        for l in range(wl.n_layers_src):
+            sk2[l, b, 2, s, 17] = bits
+            sv2[l, b, 4, s, 90] = bits
+    dirty = _run(wl, sk2, sv2, blob)
+    staged = _run(wl, sk2, sv2, blob, staged=True)
+    for c, x, y in zip(clean[:2], dirty[:2], staged[:2]):
+        for l in wl.bt_window:
+            for b, n in enumerate(wl.seq_lens):
+                for s in range(n):
+                    if any((b, s) == (bb, ss) for bb, ss, _ in bad):
+                        assert torch.isnan(x[l, b, :, s].float()).all()
+                        assert torch.isnan(y[l, b, :, s].float()).all()
+                    else:
+                        assert torch.equal(G.int_view(c[l, b, :, s]), G.int_view(x[l, b, :, s]))
