@@ -105,8 +105,9 @@ __device__ __forceinline__ void write_gate16(const PathArgs& a, int grp, size_t 
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
 
-// Grid (tiles_max, gp), 256 threads: each warp produces the gate of 16 token
-// rows of one tile for one (layer, K/V) group. Lanes split the D_s channels
+// Grid (tiles_max, gp, 16), 256 threads: each warp produces the gate of one token
+// row of one tile for one (layer, K/V) group (a warp with 16 rows leaves a short context's
+// few tiles to a handful of CTAs: 41 against 11 us for 64 fp32 tokens and 8 groups). Lanes split the D_s channels
 // (VEC-wide vectors when the head dim allows it), reduce the E logits with
 // warp shuffles, and lane 0 applies the max-subtracted softmax and the Top-K
 // renormalisation. Rows past the tile's length get a zero gate.
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(256) gate_kernel(PathArgs a) {
   const float* __restrict__ bg = a.bg + static_cast<size_t>(grp) * E;
   constexpr int NV = VEC ? Vec<T>::N : 1;
 
-  for (int r = warp; r < kTileM; r += 8) {
+  for (int r = blockIdx.z * 8 + warp; r < kTileM; r += 8 * gridDim.z) {
     float* __restrict__ gout = a.gate + (static_cast<size_t>(grp) * d.tpad + static_cast<size_t>(m) * kTileM + r) * E;
     if (r >= ti.rows) {
       if (lane < E) gout[lane] = 0.f;
@@ -413,7 +414,7 @@ cudaError_t launch_fixed_gate(const PathArgs& a, const float* fg, cudaStream_t s
 cudaError_t launch_gate(const PathArgs& a, cudaStream_t st) {
   const Dims& d = a.d;
   if (a.gp <= 0) return cudaSuccess;
-  dim3 grid(d.tiles_max, a.gp);
+  dim3 grid(d.tiles_max, a.gp), rows(d.tiles_max, a.gp, 16);   // rows: one row per warp
   // tile-wide kernel: 16-byte chunks per head row (CPR) of 8 or 16, E <= 8
   if (d.dtype == 0 && d.E <= 4 && d.d_s == 64) {
     gate_tile_kernel<__nv_bfloat16, 8, 4, 4><<<grid, 256, 0, st>>>(a);
@@ -425,14 +426,14 @@ cudaError_t launch_gate(const PathArgs& a, cudaStream_t st) {
     gate_tile_kernel<__nv_bfloat16, 16, 8, 8><<<grid, 256, 0, st>>>(a);
   } else if (d.dtype == 0) {
     if (d.d_s % 8 == 0)
-      gate_kernel<__nv_bfloat16, true><<<grid, 256, 0, st>>>(a);
+      gate_kernel<__nv_bfloat16, true><<<rows, 256, 0, st>>>(a);
     else
-      gate_kernel<__nv_bfloat16, false><<<grid, 256, 0, st>>>(a);
+      gate_kernel<__nv_bfloat16, false><<<rows, 256, 0, st>>>(a);
   } else {
     if (d.d_s % 4 == 0)
-      gate_kernel<float, true><<<grid, 256, 0, st>>>(a);
+      gate_kernel<float, true><<<rows, 256, 0, st>>>(a);
     else
-      gate_kernel<float, false><<<grid, 256, 0, st>>>(a);
+      gate_kernel<float, false><<<rows, 256, 0, st>>>(a);
   }
   return cudaGetLastError();
 }
