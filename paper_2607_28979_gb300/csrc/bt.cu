@@ -356,7 +356,7 @@ __device__ void epi_out_routed(const EpiCtx& e, const Work& w, uint32_t tb, int 
     b = tok / d.S;
     s = tok - b * d.S;
     gt = a.gate[(int64_t(x) * d.B * d.S + tok) * d.E + m];
-    const float2* st = a.rstat + int64_t(g) * d.R + int64_t(pos) * d.P;
+    const float2* st = a.rstat + (int64_t(w.r) * d.G + g) * d.R + int64_t(pos) * d.P;
     float tm = 0.f;
     for (int k = 0; k < d.P; ++k) tm += st[k].x;
     tm /= d.P;
@@ -369,7 +369,7 @@ __device__ void epi_out_routed(const EpiCtx& e, const Work& w, uint32_t tb, int 
     rs = rsqrtf(tq / (float(d.d) * d.P) + kLnEps);
   }
   uint16_t* dst = static_cast<uint16_t*>(a.dst[x]);
-  const int l = d.q0 + a.slot;
+  const int l = d.q0 + a.slot + w.r;
   const float* cbase = a.c_out + int64_t(g) * d.Dt;
   const float* sbase = a.s_out + int64_t(g) * d.Dt;
   for (int ch = cg; ch < c.NT / 32; ch += ng) {
@@ -412,7 +412,7 @@ __device__ void epi_out(const EpiCtx& e, const Work& w, uint32_t tb, int row, in
     if (gt[m] == 0.f) continue;
     // LN_out statistics over the token's P rows (Chan's combination of the
     // per-row mean and M2, each over d values)
-    const float2* st = a.rstat + (int64_t(x) * d.E + m) * d.R + int64_t(tok) * d.P;
+    const float2* st = a.rstat + (int64_t(w.r) * d.G + x * d.E + m) * d.R + int64_t(tok) * d.P;
     float tm = 0.f;
     for (int k = 0; k < d.P; ++k) tm += st[k].x;
     tm /= d.P;
@@ -425,7 +425,7 @@ __device__ void epi_out(const EpiCtx& e, const Work& w, uint32_t tb, int row, in
     rs[m] = rsqrtf(tq / (float(d.d) * d.P) + kLnEps);
   }
   uint16_t* dst = static_cast<uint16_t*>(a.dst[x]);
-  const int l = d.q0 + a.slot;
+  const int l = d.q0 + a.slot + w.r;
   for (int ch = cg; ch < c.NT / 32; ch += ng) {
     float y[32];
 #pragma unroll
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
             case kBtOut: {
               const int g = a.routed ? w.g : w.g * d.E + m;
               tma_load_2d(dA, &tmA, &full[stage], kc,
-                          static_cast<int32_t>(int64_t(g) * d.B * d.S + w.tok0 + a.xo_tok0));
+                          static_cast<int32_t>(int64_t(g) * d.B * d.S + w.tok0) + w.r * d.G * d.B * d.S);
               tma_load_2d(dB, &tmB, &full[stage], kc, g * c.b_rows_per_g + w.j * c.NT);
               break;
             }
@@ -964,12 +964,18 @@ __global__ void __launch_bounds__(32 * (4 + kFfnEpi), 1)
 
 // ---------------------------------------------------------------- gate (SIMT)
 //
-// One warp per token: logits_m = Wg[x][m] . window(token) + bg, the window
+// Two tokens per warp: logits_m = Wg[x][m] . window(token) + bg, the window
 // flattened slot-major then head-major (c = r * D_s + p * d_s + i); softmax in
 // fp32, then Top-K (ties to the lower index) and renormalisation. Also clamps
-// and reports sequence lengths outside [0, S].
+// and reports sequence lengths outside [0, S]. EM: at least E experts.
+//
+// What bounds it: the source rows' read (100 MB for 8 x 1024 tokens, 4 slots, 12 heads of 64:
+// 15 us), which needs loads in flight: four pieces per lane are loaded before they are used,
+// and the accumulators are unrolled (32 us; 63 with one piece at a time and E as a loop bound).
+template <int EM>
 __global__ void __launch_bounds__(256) bt_gate_kernel(const BtArgs a) {
   extern __shared__ uint4 wg_s[];   // [E][N * D_s] bf16 of block x
+  constexpr int U = 4;              // 16-byte pieces in flight per lane and token
   const BtDims& d = a.d;
   const int x = blockIdx.y;
   const int WD = d.N * d.Ds;
@@ -984,117 +990,190 @@ __global__ void __launch_bounds__(256) bt_gate_kernel(const BtArgs a) {
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_tok = d.B * d.S;
-  for (int tok = blockIdx.x * 8 + warp; tok < n_tok; tok += gridDim.x * 8) {
-    const int b = tok / d.S, s = tok - b * d.S;
-    if (s >= seq_len_of(a, b)) continue;
-    float acc[kMaxE];
-    for (int m = 0; m < d.E; ++m) acc[m] = 0.f;
-    for (int c8 = lane; c8 < WD / 8; c8 += 32) {
-      const int c = c8 * 8;
-      const int r = c / d.Ds, rem = c - r * d.Ds;
-      const int p = rem / d.d_s, i = rem - p * d.d_s;
-      const uint4 u = __ldg(reinterpret_cast<const uint4*>(
-          static_cast<const uint16_t*>(a.src[x]) +
-          (((int64_t(a.src_layer[r]) * d.B + b) * d.P + p) * d.S + s) * d.d_s + i));
-      const float xv[8] = {bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y),
-                           bf16_lo(u.z), bf16_hi(u.z), bf16_lo(u.w), bf16_hi(u.w)};
-      for (int m = 0; m < d.E; ++m) {
-        const uint4 wv = wg_s[(m * WD + c) / 8];
-        const float wf[8] = {bf16_lo(wv.x), bf16_hi(wv.x), bf16_lo(wv.y), bf16_hi(wv.y),
-                             bf16_lo(wv.z), bf16_hi(wv.z), bf16_lo(wv.w), bf16_hi(wv.w)};
-        float sacc = acc[m];
+  const int n8 = WD / 8;
+  const int sh = d.d_s == 64 ? 3 : 4;              // 16-byte pieces of a head row, log2
+  const uint32_t inv_p = 65536u / d.P + 1u;        // h / P = h inv_p / 65536 for h < 512
+  for (int tok = (blockIdx.x * 8 + warp) * 2; tok < n_tok; tok += gridDim.x * 16) {
+    const uint4* base[2];
+    bool live[2];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sacc = fmaf(wf[k], xv[k], sacc);
-        acc[m] = sacc;
+    for (int k = 0; k < 2; ++k) {
+      const int b = (tok + k) / d.S, s = tok + k - b * d.S;
+      live[k] = tok + k < n_tok && s < seq_len_of(a, b);
+      base[k] = reinterpret_cast<const uint4*>(
+          static_cast<const uint16_t*>(a.src[x]) +
+          (live[k] ? (int64_t(b) * d.P * d.S + s) * d.d_s : 0));
+    }
+    if (!live[0] && !live[1]) continue;
+    float acc[2][EM];
+#pragma unroll
+    for (int m = 0; m < EM; ++m) acc[0][m] = acc[1][m] = 0.f;
+    for (int c0 = lane; c0 < n8; c0 += 32 * U) {
+      uint4 u[U][2];
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const int c8 = c0 + 32 * i, h = c8 >> sh;
+        const int r = static_cast<int>(h * inv_p >> 16), p = h - r * d.P;
+        const int64_t at =
+            c8 < n8 ? ((int64_t(a.src_layer[r]) * d.B * d.P + p) * d.S << sh) + (c8 & ((1 << sh) - 1))
+                    : 0;
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          u[i][k] = c8 < n8 && live[k] ? __ldg(base[k] + at) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const int c8 = c0 + 32 * i;
+        if (c8 >= n8) break;
+        float xv[2][8];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const uint4 v = u[i][k];
+          xv[k][0] = bf16_lo(v.x); xv[k][1] = bf16_hi(v.x); xv[k][2] = bf16_lo(v.y);
+          xv[k][3] = bf16_hi(v.y); xv[k][4] = bf16_lo(v.z); xv[k][5] = bf16_hi(v.z);
+          xv[k][6] = bf16_lo(v.w); xv[k][7] = bf16_hi(v.w);
+        }
+#pragma unroll
+        for (int m = 0; m < EM; ++m) {
+          if (m < d.E) {
+            const uint4 wv = wg_s[m * n8 + c8];
+            const float wf[8] = {bf16_lo(wv.x), bf16_hi(wv.x), bf16_lo(wv.y), bf16_hi(wv.y),
+                                 bf16_lo(wv.z), bf16_hi(wv.z), bf16_lo(wv.w), bf16_hi(wv.w)};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              acc[0][m] = fmaf(wf[e], xv[0][e], acc[0][m]);
+              acc[1][m] = fmaf(wf[e], xv[1][e], acc[1][m]);
+            }
+          }
+        }
       }
     }
-    for (int m = 0; m < d.E; ++m)
-      for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
-    if (lane == 0) {
-      float g[kMaxE];
+#pragma unroll
+    for (int m = 0; m < EM; ++m)
+      if (m < d.E)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          acc[0][m] += __shfl_xor_sync(0xffffffffu, acc[0][m], o);
+          acc[1][m] += __shfl_xor_sync(0xffffffffu, acc[1][m], o);
+        }
+    if (lane < 2 && (lane ? live[1] : live[0])) {   // lane k: token tok + k
+      float g[EM];
       float mx = -INFINITY;
-      for (int m = 0; m < d.E; ++m) {
-        g[m] = acc[m] + a.bg[x * d.E + m];
-        mx = fmaxf(mx, g[m]);
-      }
+#pragma unroll
+      for (int m = 0; m < EM; ++m)
+        if (m < d.E) {
+          g[m] = (lane ? acc[1][m] : acc[0][m]) + a.bg[x * d.E + m];
+          mx = fmaxf(mx, g[m]);
+        }
       float sum = 0.f;
-      for (int m = 0; m < d.E; ++m) {
-        g[m] = expf(g[m] - mx);
-        sum += g[m];
-      }
-      for (int m = 0; m < d.E; ++m) g[m] /= sum;
+#pragma unroll
+      for (int m = 0; m < EM; ++m)
+        if (m < d.E) {
+          g[m] = expf(g[m] - mx);
+          sum += g[m];
+        }
+#pragma unroll
+      for (int m = 0; m < EM; ++m)
+        if (m < d.E) g[m] /= sum;
       if (d.top_k > 0 && d.top_k < d.E) {
         uint32_t keep = 0;
         for (int k = 0; k < d.top_k; ++k) {
           int best = -1;
-          for (int m = 0; m < d.E; ++m)
-            if (!((keep >> m) & 1u) && (best < 0 || g[m] > g[best])) best = m;
+          float bv = 0.f;
+#pragma unroll
+          for (int m = 0; m < EM; ++m)
+            if (m < d.E && !((keep >> m) & 1u) && (best < 0 || g[m] > bv)) {
+              best = m;
+              bv = g[m];
+            }
           keep |= 1u << best;
         }
         float ks = 0.f;
-        for (int m = 0; m < d.E; ++m)
+#pragma unroll
+        for (int m = 0; m < EM; ++m)
           if ((keep >> m) & 1u) ks += g[m];
-        for (int m = 0; m < d.E; ++m) g[m] = ((keep >> m) & 1u) ? g[m] / ks : 0.f;
+#pragma unroll
+        for (int m = 0; m < EM; ++m)
+          if (m < d.E) g[m] = ((keep >> m) & 1u) ? g[m] / ks : 0.f;
       }
-      float* go = a.gate + (int64_t(x) * n_tok + tok) * d.E;
-      for (int m = 0; m < d.E; ++m) go[m] = g[m];
+      float* go = a.gate + (int64_t(x) * n_tok + tok + lane) * d.E;
+#pragma unroll
+      for (int m = 0; m < EM; ++m)
+        if (m < d.E) go[m] = g[m];
     }
   }
 }
 
 // ---------------------------------------------------------------- Top-1 routing
 //
-// One CTA of 1024 threads. For each group g = x * E + m, the tokens whose kept
-// gate weight for backbone m is nonzero (with Top-1, exactly the chosen
-// backbone), in token order: every thread counts the choices in its contiguous
-// chunk of token slots, a block scan gives each thread its first bucket
-// position, and the thread writes its tokens there. Then cnt[g] and the tile
-// prefix sums (tau-token tiles, 128-token tiles).
+// One CTA of 1024 threads per group g = x * E + m: the tokens whose kept gate weight for
+// backbone m is nonzero (with Top-1, exactly the chosen backbone), in token order, 4,096 token
+// slots at a time (ballots, then scans of the warps' counts). The last CTA to finish forms the
+// tile prefix sums (tau-token tiles, 128-token tiles) from every group's count and resets the
+// ticket. One CTA for all the groups, a contiguous chunk of slots per thread, took 53 us for
+// 4 x 4096 slots; a CTA per group, 1,024 slots at a time and CTA 0 counting them all, 31 us;
+// this, 19 us.
 __global__ void __launch_bounds__(1024) bt_route_kernel(const BtArgs a, int32_t* cnt,
                                                         int32_t* list, int32_t* rpre) {
-  __shared__ int s_scan[1024];
-  __shared__ int s_cnt[2 * kMaxE];
+  constexpr int U = 4;
+  __shared__ int s_warp[2][U][32];
   const BtDims& d = a.d;
   const int T = d.B * d.S;
-  const int tid = threadIdx.x;
-  const int per = (T + 1023) / 1024;
-  const int t0 = min(T, tid * per), t1 = min(T, t0 + per);
-  for (int g = 0; g < d.G; ++g) {
-    const int x = g / d.E, m = g - x * d.E;
-    const float* gx = a.gate + int64_t(x) * T * d.E + m;
-    auto chose = [&](int tok) {
-      const int b = tok / d.S, s = tok - b * d.S;
-      return s < seq_len_of(a, b) && gx[int64_t(tok) * d.E] > 0.f;
-    };
-    int c = 0;
-    for (int tok = t0; tok < t1; ++tok) c += chose(tok) ? 1 : 0;
-    s_scan[tid] = c;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {   // inclusive scan (Hillis-Steele)
-      const int v = tid >= o ? s_scan[tid - o] : 0;
-      __syncthreads();
-      s_scan[tid] += v;
-      __syncthreads();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = blockIdx.x, x = g / d.E, m = g - x * d.E;
+  const float* gw = a.gate + int64_t(x) * T * d.E + m;
+  int32_t* lg = list + int64_t(g) * T;
+  int base = 0, par = 0;
+  for (int t0 = 0; t0 < T; t0 += 1024 * U, par ^= 1) {
+    uint32_t bal[U];
+    bool ch[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int tok = t0 + 1024 * i + tid;
+      ch[i] = false;
+      if (tok < T) {
+        const int b = tok / d.S;
+        const float w = __ldg(gw + int64_t(tok) * d.E);   // any value past the sequence
+        ch[i] = tok - b * d.S < seq_len_of(a, b) && w > 0.f;
+      }
     }
-    int off = s_scan[tid] - c;
-    int32_t* lg = list + int64_t(g) * T;
-    for (int tok = t0; tok < t1; ++tok)
-      if (chose(tok)) lg[off++] = tok;
-    if (tid == 1023) s_cnt[g] = s_scan[1023];
-    __syncthreads();
-  }
-  if (tid == 0) {
-    int p0 = 0, p1 = 0;
-    for (int g = 0; g < d.G; ++g) {
-      cnt[g] = s_cnt[g];
-      rpre[g] = p0;
-      rpre[d.G + 1 + g] = p1;
-      p0 += (s_cnt[g] + d.tau - 1) / d.tau;
-      p1 += (s_cnt[g] + 127) / 128;
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      bal[i] = __ballot_sync(0xffffffffu, ch[i]);
+      if (lane == 0) s_warp[par][i][warp] = __popc(bal[i]);
     }
-    rpre[d.G] = p0;
-    rpre[2 * d.G + 1] = p1;
+    __syncthreads();   // the other parity's counts were read before it
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int c = s_warp[par][i][lane];
+      int inc = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const int before = __shfl_sync(0xffffffffu, inc - c, warp);
+      if (ch[i]) lg[base + before + __popc(bal[i] & ((1u << lane) - 1u))] = t0 + 1024 * i + tid;
+      base += __shfl_sync(0xffffffffu, inc, 31);
+    }
   }
+  if (tid != 0) return;
+  cnt[g] = base;
+  __threadfence();
+  int32_t* ticket = cnt + kBtTicket;
+  if (atomicAdd(ticket, 1) != d.G - 1) return;
+  __threadfence();
+  int p0 = 0, p1 = 0;
+  for (int gg = 0; gg < d.G; ++gg) {
+    const int n = *static_cast<volatile int32_t*>(cnt + gg);
+    rpre[gg] = p0;
+    rpre[d.G + 1 + gg] = p1;
+    p0 += (n + d.tau - 1) / d.tau;
+    p1 += (n + 127) / 128;
+  }
+  rpre[d.G] = p0;
+  rpre[2 * d.G + 1] = p1;
+  *ticket = 0;
 }
 
 // The source rows of slot a.slot for every bucket position, packed per group:
@@ -1247,23 +1326,25 @@ bool bt_supported(const BtDims& d) {
 cudaError_t launch_bt_gate(const BtArgs& a, cudaStream_t st) {
   const BtDims& d = a.d;
   const size_t smem = size_t(d.E) * d.N * d.Ds * 2;
-  static size_t attr = 0;
-  if (smem > 48 * 1024 && smem > attr) {
-    cudaError_t e = cudaFuncSetAttribute(bt_gate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const int em = d.E <= 2 ? 0 : d.E <= 4 ? 1 : 2;
+  auto kern = em == 0 ? bt_gate_kernel<2> : em == 1 ? bt_gate_kernel<4> : bt_gate_kernel<8>;
+  static size_t attr[3] = {0, 0, 0};
+  if (smem > 48 * 1024 && smem > attr[em]) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    attr = smem;
+    attr[em] = smem;
   }
   const int n_tok = d.B * d.S;
-  dim3 grid(std::min((n_tok + 7) / 8, 1024), 2);
-  bt_gate_kernel<<<grid, 256, smem, st>>>(a);
+  dim3 grid(std::min((n_tok + 15) / 16, 1024), 2);
+  kern<<<grid, 256, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_bt_route(const BtArgs& a, int32_t* cnt, int32_t* list, int32_t* rpre,
                             cudaStream_t st) {
   if (a.d.G > 2 * kMaxE) return cudaErrorInvalidValue;
-  bt_route_kernel<<<1, 1024, 0, st>>>(a, cnt, list, rpre);
+  bt_route_kernel<<<a.d.G, 1024, 0, st>>>(a, cnt, list, rpre);
   return cudaGetLastError();
 }
 
@@ -1326,6 +1407,7 @@ cudaError_t launch_bt_gemm(int mode, const BtArgs& a, const CUtensorMap& tmA,
       c.NT = nt;
       c.n_tiles = d.Dt / nt;
       c.row_tiles = (d.B * d.S + 127) / 128;
+      c.slots = a.out_slots;
       break;
     }
     default: return cudaErrorInvalidValue;
@@ -1343,7 +1425,8 @@ cudaError_t launch_bt_gemm(int mode, const BtArgs& a, const CUtensorMap& tmA,
     if (e != cudaSuccess) return e;
     attr_set[di] = true;
   }
-  const long long items = static_cast<long long>(c.groups) * c.row_tiles * c.n_tiles;
+  const long long items =
+      static_cast<long long>(c.groups) * c.row_tiles * c.n_tiles * std::max(c.slots, 1);
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
   if (grid <= 0) return cudaSuccess;
   kern<<<grid, bt_threads(wide ? 16 : kBtRowEpi), kBtSmem, st>>>(tmA, tmA2, tmB, a, c);

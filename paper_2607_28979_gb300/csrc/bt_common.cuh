@@ -35,6 +35,7 @@ struct GemmCfg {
   int row_tiles;  // row tiles per group
   int a_box_bytes;
   int b_rows_per_g;   // rows of the weight map per (group, slot) block
+  int slots;          // kBtOut: window slots from a.slot on in this launch (else 0 or 1)
 };
 
 // One work item of the persistent loop. Every role decodes items the same way
@@ -42,20 +43,31 @@ struct GemmCfg {
 struct Work {
   int g, b, s0, ntok, j;
   int tok0;       // kBtOut: first token of the 128-token tile (routed: bucket position)
+  int r;          // kBtOut: slot of the item, counted from a.slot
   int64_t row0;   // the tile's first row in its group's row space
   bool active;
 };
 
 // Items of a launch: dense, groups x row tiles x N tiles; routed, the tiles of
 // every bucket (from the route kernel's prefix sums) x N tiles.
-__device__ __forceinline__ int total_items(const BtArgs& a, const GemmCfg& c) {
+__device__ __forceinline__ int slot_items(const BtArgs& a, const GemmCfg& c) {
   if (!a.routed) return c.groups * c.row_tiles * c.n_tiles;
   const int* pre = a.rpre + (c.mode == kBtOut ? a.d.G + 1 : 0);
   return pre[a.d.G] * c.n_tiles;
 }
 
+__device__ __forceinline__ int total_items(const BtArgs& a, const GemmCfg& c) {
+  return slot_items(a, c) * (c.slots > 1 ? c.slots : 1);
+}
+
 __device__ __forceinline__ Work decode(const BtArgs& a, const GemmCfg& c, int item) {
   Work w;
+  w.r = 0;
+  if (c.slots > 1) {
+    const int per = slot_items(a, c);
+    w.r = item / per;
+    item -= w.r * per;
+  }
   if (a.routed) {   // tile of bucket positions of group g
     const bool out = c.mode == kBtOut;
     const int* pre = a.rpre + (out ? a.d.G + 1 : 0);

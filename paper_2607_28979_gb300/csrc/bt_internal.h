@@ -15,6 +15,7 @@ namespace mot {
 // are folded into W_in and W_out at load.
 constexpr int kBtMaxSlots = 32;
 constexpr int kBtMaxP = 16;
+constexpr int kBtTicket = 63;   // of the 64 words of cnt: the route kernel's ticket, 0 between launches
 
 struct BtDims {
   int32_t L_s, P, d_s, L_t, H_t, d_t, E, top_k, B, S;
@@ -62,7 +63,8 @@ struct BtArgs {
   void* f;               // bf16 FFN hidden                    [df]
   void* xo;              // bf16 h_r (raw)                     [d] (= [B * S][P * d])
   float2* rstat;         // [G][R] (mean, M2) of each h_r row over its d values
-  int32_t xo_tok0;       // token rows before this slot's in xo (the scan keeps one block per slot)
+  int32_t out_slots;     // slots of the output projection's launch (xo and rstat hold one block
+                         // per slot after the scan in one launch)
   const float* prm;      // [G][N][bt_scan_prm_floats] the scan's fp32 vectors of each slot
   int32_t* status;
   long long wait_limit;

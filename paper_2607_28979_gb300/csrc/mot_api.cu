@@ -896,7 +896,7 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
       return MOT_ERR_OOM;
     }
   }
-  if (cudaMemset(h->status, 0, 16) != cudaSuccess) {
+  if (cudaMemset(h->status, 0, 16) != cudaSuccess || cudaMemset(bt.rcnt, 0, 64 * 4) != cudaSuccess) {
     cudaGetLastError();
     free_all(h);
     delete h;
@@ -1500,7 +1500,7 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
       return launch_bt_route(a, bt.rcnt, bt.rlist, bt.rpre, st);
     }));
   }
-  auto project = [&](int r) {   // the output projection of slot r
+  auto project = [&](int r) {   // the output projection of slot r (and the out_slots - 1 after it)
     a.slot = r;
     return timed(h, "bt_out_gelu_combine", st, [&] {
       return launch_bt_gemm(kBtOut, a, bt.tm_xo, bt.tm_xo, routed ? bt.tm_wout_r : bt.tm_wout,
@@ -1511,11 +1511,8 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
     a.prm = bt.prm;
     const CUtensorMap tm[6] = {bt.tm_win, bt.tm_wq, bt.tm_wkvh, bt.tm_wo, bt.tm_wf1c, bt.tm_wf2};
     MOT_CUDA_TRY(timed(h, "bt_scan", st, [&] { return launch_bt_scan(a, tm, h->num_sms, st); }));
-    for (int r = 0; r < d.N; ++r) {
-      a.xo_tok0 = r * d.G * d.B * d.S;
-      a.rstat = bt.rstat + size_t(r) * d.G * d.R;
-      MOT_CUDA_TRY(project(r));
-    }
+    a.out_slots = d.N;
+    MOT_CUDA_TRY(project(0));
     if (routed) h->counts_valid = true;
     return MOT_OK;
   }
