@@ -3,6 +3,7 @@
 #include <cuda_fp16.h>
 
 #include "mot_internal.h"
+#include "ptx.cuh"
 
 namespace mot {
 
@@ -14,6 +15,7 @@ namespace mot {
 __global__ void prep_tiles_kernel(const int32_t* __restrict__ seq_lens, int32_t batch, int32_t S,
                                   TileInfo* __restrict__ tiles, int32_t* __restrict__ n_tiles,
                                   int32_t* __restrict__ status) {
+  pdl_enter();
   __shared__ int32_t s_len[4096];
   __shared__ int32_t s_off[4096];
   for (int b = threadIdx.x; b < batch; b += blockDim.x) {
@@ -116,6 +118,7 @@ __global__ void __launch_bounds__(256) gate_kernel(PathArgs a) {
   const Dims& d = a.d;
   const int m = blockIdx.x;
   const int grp = a.g0 + blockIdx.y;
+  pdl_enter();
   if (m >= *a.n_tiles) return;
   const TileInfo ti = a.tiles[m];
   const GroupInfo gi = a.groups[grp];
@@ -229,6 +232,7 @@ __global__ void __launch_bounds__(256) gate_tile_kernel(PathArgs a) {
   const Dims& d = a.d;
   const int m = blockIdx.x;
   const int grp = a.g0 + blockIdx.y;
+  pdl_enter();
   if (m >= *a.n_tiles) return;
   const TileInfo ti = a.tiles[m];
   const GroupInfo gi = a.groups[grp];
@@ -388,6 +392,7 @@ __global__ void __launch_bounds__(kTileM) fixed_gate_kernel(PathArgs a, const fl
   const Dims& d = a.d;
   const int m = blockIdx.x;
   const int grp = a.g0 + blockIdx.y;
+  pdl_enter();
   if (m >= *a.n_tiles) return;
   const TileInfo ti = a.tiles[m];
   const int r = threadIdx.x;
@@ -417,23 +422,23 @@ cudaError_t launch_gate(const PathArgs& a, cudaStream_t st) {
   dim3 grid(d.tiles_max, a.gp), rows(d.tiles_max, a.gp, 16);   // rows: one row per warp
   // tile-wide kernel: 16-byte chunks per head row (CPR) of 8 or 16, E <= 8
   if (d.dtype == 0 && d.E <= 4 && d.d_s == 64) {
-    gate_tile_kernel<__nv_bfloat16, 8, 4, 4><<<grid, 256, 0, st>>>(a);
+    return launch_kernel(a.overlap, gate_tile_kernel<__nv_bfloat16, 8, 4, 4>, grid, 256, 0, st, a);
   } else if (d.dtype == 0 && d.E <= 8 && d.d_s == 64) {
-    gate_tile_kernel<__nv_bfloat16, 8, 4, 8><<<grid, 256, 0, st>>>(a);
+    return launch_kernel(a.overlap, gate_tile_kernel<__nv_bfloat16, 8, 4, 8>, grid, 256, 0, st, a);
   } else if (d.dtype == 0 && d.E <= 4 && d.d_s == 128) {
-    gate_tile_kernel<__nv_bfloat16, 16, 8, 4><<<grid, 256, 0, st>>>(a);
+    return launch_kernel(a.overlap, gate_tile_kernel<__nv_bfloat16, 16, 8, 4>, grid, 256, 0, st, a);
   } else if (d.dtype == 0 && d.E <= 8 && d.d_s == 128) {
-    gate_tile_kernel<__nv_bfloat16, 16, 8, 8><<<grid, 256, 0, st>>>(a);
+    return launch_kernel(a.overlap, gate_tile_kernel<__nv_bfloat16, 16, 8, 8>, grid, 256, 0, st, a);
   } else if (d.dtype == 0) {
     if (d.d_s % 8 == 0)
-      gate_kernel<__nv_bfloat16, true><<<rows, 256, 0, st>>>(a);
+      return launch_kernel(a.overlap, gate_kernel<__nv_bfloat16, true>, rows, 256, 0, st, a);
     else
-      gate_kernel<__nv_bfloat16, false><<<rows, 256, 0, st>>>(a);
+      return launch_kernel(a.overlap, gate_kernel<__nv_bfloat16, false>, rows, 256, 0, st, a);
   } else {
     if (d.d_s % 4 == 0)
-      gate_kernel<float, true><<<rows, 256, 0, st>>>(a);
+      return launch_kernel(a.overlap, gate_kernel<float, true>, rows, 256, 0, st, a);
     else
-      gate_kernel<float, false><<<rows, 256, 0, st>>>(a);
+      return launch_kernel(a.overlap, gate_kernel<float, false>, rows, 256, 0, st, a);
   }
   return cudaGetLastError();
 }

@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_slot;
+  pdl_enter();
 
   const int n_m = min(*p.n_tiles, d.tiles_max);
   const int total = p.gp * n_m;
@@ -285,8 +286,7 @@ cudaError_t launch_gate_mma(const PathArgs& a, const CUtensorMap& tmK, const CUt
   const long long items = static_cast<long long>(a.gp) * a.d.tiles_max;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
   if (grid <= 0) return cudaSuccess;
-  gate_mma_kernel<<<grid, kGThreads, kGSmem, st>>>(tmK, tmV, tmWg, a);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, gate_mma_kernel, grid, kGThreads, kGSmem, st, tmK, tmV, tmWg, a);
 }
 
 }  // namespace mot

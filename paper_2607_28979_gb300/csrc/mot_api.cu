@@ -367,6 +367,7 @@ mot_status run_translate(mot_ctx* h, const void* src_k, const void* src_v, const
     MOT_CUDA_TRY(timed(h, "prep_tiles", st, [&] {
       return launch_prep(seq_lens, batch, d, h->tiles, h->n_tiles, h->status, st);
     }));
+  a.overlap = do_prep && !h->profile;   // behind the tile list; the kernels after the gate, always
   a.g0 = g_begin;
   a.gp = g_end - g_begin;
   const bool routed = h->use_umma && h->sparse_ok && h->routing == 1;
@@ -380,6 +381,7 @@ mot_status run_translate(mot_ctx* h, const void* src_k, const void* src_v, const
                          : launch_gate(a, st);
     }));
   }
+  a.overlap = !h->profile;
   if (routed) {   // Top-K: per-expert token buckets, passes of gp_sparse groups
     const SparseArgs& sp = h->sp;
     for (int g0 = g_begin; g0 < g_end; g0 += h->gp_sparse) {
@@ -1426,6 +1428,7 @@ mot_status mot_translate_h(mot_handle h, const void* src_act, const int32_t* seq
     a.dst[0] = dst_k;
     a.dst[1] = dst_v;
     a.proj_layer = h->proj_layer;
+    a.overlap = !h->profile;
     a.g0 = g0;
     a.gp = g1 - g0;
     MOT_CUDA_TRY(timed(h, "umma2_proj", st, [&] {
@@ -1496,6 +1499,7 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
     a.list = bt.rlist;
     a.rpre = bt.rpre;
     a.xs = bt.xs;
+    a.overlap = !h->profile;
     MOT_CUDA_TRY(timed(h, "bt_route", st, [&] {
       return launch_bt_route(a, bt.rcnt, bt.rlist, bt.rpre, st);
     }));
@@ -1509,6 +1513,7 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
   };
   if (bt.scan && !h->profile) {   // profiling times the stages one by one
     a.prm = bt.prm;
+    a.overlap = true;
     const CUtensorMap tm[6] = {bt.tm_win, bt.tm_wq, bt.tm_wkvh, bt.tm_wo, bt.tm_wf1c, bt.tm_wf2};
     MOT_CUDA_TRY(timed(h, "bt_scan", st, [&] { return launch_bt_scan(a, tm, h->num_sms, st); }));
     a.out_slots = d.N;
@@ -1672,6 +1677,7 @@ mot_status mot_replay_attention(mot_handle h, int32_t layer, const void* q, cons
     if (!encode_bf16(&tmK, k, 2, kd, ks, box) || !encode_bf16(&tmVt, h->rvt, 2, vd, vs, vbox))
       return MOT_ERR_CUDA;
     MOT_CUDA_TRY(timed(h, "replay_vt", st, [&] { return launch_replay_vt(a, h->rvt, st); }));
+    a.overlap = !h->profile;
     MOT_CUDA_TRY(timed(h, "replay_fmha_full", st,
                        [&] { return launch_replay_fmha(a, tmK, tmVt, st); }));
     return MOT_OK;
@@ -1680,6 +1686,7 @@ mot_status mot_replay_attention(mot_handle h, int32_t layer, const void* q, cons
   // the tensor-core tiling does not take, over the rows 0..u
   if (!full)
     MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, h->num_sms, st); }));
+  a.overlap = !full && !h->profile;
   MOT_CUDA_TRY(timed(h, full ? "replay_attn_full" : "replay_attn_sparse", st,
                      [&] { return launch_replay_gather(a, h->num_sms, st); }));
   return MOT_OK;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "mot.h"
 
 #include <nvtx3/nvToolsExt.h>
@@ -20,6 +22,28 @@ struct NvtxRange {
   NvtxRange(const NvtxRange&) = delete;
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
+
+// Launch `kernel`; with `overlap` it may start before the stream's preceding kernel has
+// finished (programmatic stream serialization). Only for a kernel that calls pdl_enter before
+// it touches what others write, directly behind a kernel of the same call: each kernel of the
+// chain then waits for the one before it, so a chain completes in order. The launch and
+// prologue of a kernel (barriers, tensor-memory allocation, descriptors) hide behind its
+// predecessor's last CTAs.
+template <class... P, class... A>
+cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 constexpr int kTileM = 128;   // tokens per token tile (rows of one MMA tile)
 constexpr int kMaxE = 16;     // translators per (layer, K/V) group
@@ -85,6 +109,7 @@ struct PathArgs {
   int32_t g0, gp;         // groups [g0, g0 + gp) of this pass
   long long wait_limit;   // bound of every pipeline wait, in SM cycles
   int32_t stall_test;     // test hook (single-SM GEMM1): CTA 0 withholds its first stage
+  bool overlap;           // this launch may overlap the kernel before it (launch_kernel)
 };
 
 // Top-K routing (0 < top_k < E) on the tensor-core path (sparse.cu): for each

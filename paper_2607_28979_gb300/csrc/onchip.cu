@@ -199,6 +199,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = bars->tmem_slot;
+  pdl_enter();
 
   const int n_m = min(*p.n_tiles, d.tiles_max);
   const int n_mp = (n_m + 1) / 2;
@@ -549,8 +550,8 @@ cudaError_t launch_onchip(const PathArgs& a, const CUtensorMap& tmK, const CUten
   const long long max_pairs = num_sms / 2;
   const int grid = 2 * static_cast<int>(pairs < max_pairs ? pairs : max_pairs);
   if (grid <= 0) return cudaSuccess;
-  onchip_kernel<<<grid, kThreads, kSmemBytes, st>>>(tmK, tmV, tmW1q, tmW2h, tmG16, tmB2th, oa);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, onchip_kernel, grid, kThreads, kSmemBytes, st, tmK, tmV, tmW1q, tmW2h,
+                       tmG16, tmB2th, oa);
 }
 
 }  // namespace mot

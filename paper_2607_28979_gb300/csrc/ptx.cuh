@@ -105,6 +105,16 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// ---------------------------------------------------------------- dependent launches
+//
+// pdl_enter: let the next kernel of the stream start its prologue as SMs come free, and wait
+// until the kernel before this one (if this launch may overlap it) has finished and its writes
+// are visible. Everything before it touches nothing that another kernel writes.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- cp.async (16-byte copies)
 
 // One 16-byte global -> shared copy (L2 only, not L1), tracked by commit groups.

@@ -99,6 +99,7 @@ __device__ __forceinline__ void pad_row(const ReplayArgs& a, int32_t* out) {
 // Each lane reads 8 consecutive scores per step (16-byte loads when max_seq % 8
 // == 0); every pass reads the row again.
 __global__ void __launch_bounds__(32 * kSelWarps) replay_select_stream_kernel(const ReplayArgs a) {
+  pdl_enter();
   __shared__ int hist[kSelWarps][kSelCopies][256];   // copy lane % kSelCopies: fewer same-bin collisions
   const ReplayDims& d = a.d;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -206,6 +207,7 @@ constexpr int kSelCacheRounds = 16;  // 256-position rounds cached per row: max_
 constexpr int kSelCacheCopies = 1;   // histogram copies per warp (36 KB per CTA: 6 CTAs per SM)
 
 __global__ void __launch_bounds__(32 * kSelCacheWarps) replay_select_hist_kernel(const ReplayArgs a) {
+  pdl_enter();
   __shared__ int hist[kSelCacheWarps][kSelCacheCopies][256];   // copy lane % kSelCacheCopies
   __shared__ uint4 keys[kSelCacheWarps][kSelCacheRounds][32];
   const ReplayDims& d = a.d;
@@ -727,6 +729,7 @@ __device__ __forceinline__ bool select_bounded(const RowWords& rw, uint16_t* lis
 template <int SETS>
 __global__ void __launch_bounds__(32 * kSelRowWarps, kSelRowCtas)
     replay_select_kernel(const ReplayArgs a) {
+  pdl_enter();
   constexpr int CAP = 512 * SETS;
   __shared__ uint16_t lists[kSelRowWarps][CAP];   // candidate slots, ascending
   const ReplayDims& d = a.d;
@@ -758,6 +761,7 @@ __global__ void __launch_bounds__(32 * kSelRowWarps, kSelRowCtas)
 // 4 x 4096 positions and 2 heads of 128 in 9.2 us (15.6 us with one value per thread and step).
 __global__ void __launch_bounds__(256) replay_vt_kernel(const uint16_t* __restrict__ v,
                                                          uint16_t* __restrict__ vt, int N, int D) {
+  pdl_enter();
   constexpr int kLd = 66;   // rows of 33 words: a column of words in 32 banks
   __shared__ __align__(4) uint16_t tile[64 * kLd];   // [i][j]
   const int bh = blockIdx.z;

@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(Fa<D>::kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_enter();
   const uint32_t tmem = *tmem_slot;
   uint32_t issued_mask = 0, issue_parity = 0;
   bool mma_issued = false;
@@ -539,7 +540,6 @@ cudaError_t launch_replay_fmha(const ReplayArgs& a, const CUtensorMap& tmK,
     attr[di] = true;
   }
   const int n_qt = (d.N + 127) / 128;
-  kern<<<d.B * d.Hq * n_qt, Fa<128>::kThreads, smem, st>>>(tmK, tmVt, a);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, kern, d.B * d.Hq * n_qt, Fa<128>::kThreads, smem, st, tmK, tmVt, a);
 }
 }  // namespace mot

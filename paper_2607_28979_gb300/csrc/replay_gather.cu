@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
   constexpr int MT = CH / 16, DT = D / 16, TPC = CH / C::kRows, MPT = C::kRows / 16;
   static_assert(TPC >= 2 && (2 * TPC) % kRgStages == 0, "tile stream");
   extern __shared__ uint8_t smem_raw[];
+  pdl_enter();
   const ReplayDims& d = a.d;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
@@ -474,8 +475,7 @@ cudaError_t launch_gather(const ReplayArgs& a, int num_sms, cudaStream_t st) {
   }
   const int64_t items = int64_t(a.d.B) * a.d.Hkv * a.d.N;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);   // persistent
-  kernel<<<grid, 32 * C::kWarps, C::kSmem, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, kernel, grid, 32 * C::kWarps, C::kSmem, st, a);
 }
 
 // Sets of one unit (guided, S <= 128).

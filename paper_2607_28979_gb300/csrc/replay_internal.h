@@ -31,6 +31,7 @@ struct ReplayArgs {
   int32_t full;   // 1: attend to every position 0..u
   int32_t* status;
   long long wait_limit;   // bound of every pipeline wait (SM cycles)
+  bool overlap;           // this launch may overlap the kernel before it (launch_kernel)
   int32_t stall_test;     // test hook: the gather kernel's first CTA waits for a signal nothing sends
 };
 bool replay_supported(const ReplayDims& d);

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
   float* sm = reinterpret_cast<float*>(simt_smem4);
   const Dims& d = a.d;
   const int m = blockIdx.x >> 1;
+  pdl_enter();
   if (m >= *a.n_tiles) return;
   const TileInfo ti = a.tiles[m];
   const int row0 = (blockIdx.x & 1) * BM;   // row offset inside the 128-row tile
@@ -243,8 +244,7 @@ cudaError_t launch_simt_v(const PathArgs& a, cudaStream_t st) {
   }
   const int N = GEMM == 1 ? d.EH : d.Dt;
   dim3 grid(2 * d.tiles_max, (N + BN - 1) / BN, a.gp);
-  simt_gemm_kernel<T, GEMM, VEC><<<grid, kSimtThreads, kSimtSmem, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, simt_gemm_kernel<T, GEMM, VEC>, grid, kSimtThreads, kSimtSmem, st, a);
 }
 
 template <typename T, int GEMM>

@@ -199,6 +199,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(threads2(MODE), 1)
   cluster_sync();   // barrier inits and the TMEM address are visible in both CTAs
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_enter();
 
   const int n_m = min(*p.n_tiles, d.tiles_max);
   const int n_mp = (n_m + 1) / 2;
@@ -447,9 +448,8 @@ cudaError_t launch_umma2(const PathArgs& a, const SparseArgs* sp, const CUtensor
   const long long max_pairs = num_sms / 2;
   const int grid = 2 * static_cast<int>(pairs < max_pairs ? pairs : max_pairs);
   if (grid <= 0) return cudaSuccess;
-  umma2_gemm_kernel<MODE, SPARSE>
-      <<<grid, threads2(MODE), smem_bytes2(MODE), st>>>(A0, A1, B, S, ua);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, umma2_gemm_kernel<MODE, SPARSE>, grid, threads2(MODE),
+                       smem_bytes2(MODE), st, A0, A1, B, S, ua);
 }
 
 }  // namespace
