@@ -509,7 +509,6 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_enter();
 
   const int total = total_items(a, c);
   uint32_t issued_mask = 0, issue_parity = 0;
@@ -976,7 +975,6 @@ __global__ void __launch_bounds__(32 * (4 + kFfnEpi), 1)
 template <int EM>
 __global__ void __launch_bounds__(256) bt_gate_kernel(const BtArgs a) {
   extern __shared__ uint4 wg_s[];   // [E][N * D_s] bf16 of block x
-  pdl_enter();
   constexpr int U = 4;              // 16-byte pieces in flight per lane and token
   const BtDims& d = a.d;
   const int x = blockIdx.y;
@@ -1119,7 +1117,6 @@ __global__ void __launch_bounds__(1024) bt_route_kernel(const BtArgs a, int32_t*
                                                         int32_t* list, int32_t* rpre) {
   constexpr int U = 4;
   __shared__ int s_warp[2][U][32];
-  pdl_enter();
   const BtDims& d = a.d;
   const int T = d.B * d.S;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1347,7 +1344,8 @@ cudaError_t launch_bt_gate(const BtArgs& a, cudaStream_t st) {
 cudaError_t launch_bt_route(const BtArgs& a, int32_t* cnt, int32_t* list, int32_t* rpre,
                             cudaStream_t st) {
   if (a.d.G > 2 * kMaxE) return cudaErrorInvalidValue;
-  return launch_kernel(a.overlap, bt_route_kernel, a.d.G, 1024, 0, st, a, cnt, list, rpre);
+  bt_route_kernel<<<a.d.G, 1024, 0, st>>>(a, cnt, list, rpre);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_bt_pack(const BtArgs& a, void* xs, cudaStream_t st) {
@@ -1431,8 +1429,8 @@ cudaError_t launch_bt_gemm(int mode, const BtArgs& a, const CUtensorMap& tmA,
       static_cast<long long>(c.groups) * c.row_tiles * c.n_tiles * std::max(c.slots, 1);
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
   if (grid <= 0) return cudaSuccess;
-  return launch_kernel(a.overlap, kern, grid, bt_threads(wide ? 16 : kBtRowEpi), kBtSmem, st, tmA, tmA2,
-                       tmB, a, c);
+  kern<<<grid, bt_threads(wide ? 16 : kBtRowEpi), kBtSmem, st>>>(tmA, tmA2, tmB, a, c);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_bt_ffn(const BtArgs& a, const CUtensorMap& tmXf, const CUtensorMap& tmW1,

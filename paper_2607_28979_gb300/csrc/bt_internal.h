@@ -68,7 +68,6 @@ struct BtArgs {
   const float* prm;      // [G][N][bt_scan_prm_floats] the scan's fp32 vectors of each slot
   int32_t* status;
   long long wait_limit;
-  bool overlap;          // this launch may overlap the kernel before it (launch_kernel)
   // Top-1 routing (token buckets): group g's row space holds only the tokens
   // that chose backbone g % E, packed in token order: row (pos * P + p) for
   // bucket position pos < cnt[g], whose token slot b * S + s is list[g][pos].

@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(kScThreads, 1)
   constexpr int D = kScD, DS = 16 * NXV;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_hc = d.df / 128;
+  const int total = total_items(a, c);
   const long long wl = a.wait_limit;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kScMaxRing; ++s) {
@@ -217,8 +218,6 @@ __global__ void __launch_bounds__(kScThreads, 1)
   __syncthreads();
   tc_fence_after();
   const int prm_bytes = prm_floats(d.df) * 4;
-  pdl_enter();
-  const int total = total_items(a, c);
   const uint32_t tmem = *tmem_slot;   // h at 0, accumulators at 128, 256 and 384
   uint32_t issued_mask = 0, issue_parity = 0, prm_issued = 0, prm_parity = 0;
   bool mma_issued = false;
@@ -772,8 +771,9 @@ cudaError_t launch_scan(const BtArgs& a, const CUtensorMap (&tm)[6], int num_sms
   const long long items = static_cast<long long>(c.groups) * c.row_tiles;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
   if (grid <= 0) return cudaSuccess;
-  return launch_kernel(a.overlap, kern, grid, kScThreads, at + n_ring * kScBlk + 1024, st, tm[0], tm[1],
-                       tm[2], tm[3], tm[4], tm[5], a, c, n_ring, at);
+  kern<<<grid, kScThreads, at + n_ring * kScBlk + 1024, st>>>(tm[0], tm[1], tm[2], tm[3], tm[4],
+                                                              tm[5], a, c, n_ring, at);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -806,7 +806,7 @@ void bt_scan_pack_prm(const BtDims& d, const BtScanVecs& v, int g, int slot, flo
 }
 
 // Rows of 128 (one 128-column tile of state), an FFN in whole 128-column chunks whose vectors
-// leave room for the ring (d_f up to about 3,500), and a window of at most 16 slots (the state
+// leave room for the ring (d_f up to 4,096), and a window of at most 16 slots (the state
 // rows of every slot are kept for the output projections).
 bool bt_scan_supported(const BtDims& d) {
   return d.d == kScD && d.df % 128 == 0 && d.df <= 4096 && ring_blocks(d.df) >= kScMinRing &&

@@ -28,7 +28,11 @@ struct NvtxRange {
 // it touches what others write, directly behind a kernel of the same call: each kernel of the
 // chain then waits for the one before it, so a chain completes in order. The launch and
 // prologue of a kernel (barriers, tensor-memory allocation, descriptors) hide behind its
-// predecessor's last CTAs.
+// predecessor's last CTAs, which matters where kernels are short: 57.6 -> 53.0 us for a 64-token
+// mixture of 24 x 128 x 128 blocks, 121 -> 114.7 us for 64 tokens in fp32. Tensor memory is
+// allocated before pdl_enter, so no dependent can hold what its predecessor still waits for.
+// Not used by the Top-K passes (their waiting CTAs hold back the pack and combine kernels:
+// 3.41 -> 3.45 ms) nor by the backbone chain (no gain).
 template <class... P, class... A>
 cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                           cudaStream_t st, A&&... args) {

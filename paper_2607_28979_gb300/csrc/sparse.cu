@@ -19,7 +19,6 @@
 #include <algorithm>
 
 #include "mot_internal.h"
-#include "ptx.cuh"
 
 namespace mot {
 namespace {
@@ -76,7 +75,6 @@ __device__ __forceinline__ int block_scan_flag(int f, int* s_warp, int* total) {
 
 // grid (gp, E): tokens of bucket (local group, expert).
 __global__ void __launch_bounds__(kRouteThreads) route_count_kernel(PathArgs a, SparseArgs s) {
-  pdl_enter();
   const int g = blockIdx.x, m = blockIdx.y, grp = a.g0 + g, E = a.d.E;
   const int n_rows = n_rows_of(a);
   const uint32_t* __restrict__ sel = a.sel + static_cast<size_t>(grp) * a.d.tpad;
@@ -100,7 +98,6 @@ __global__ void __launch_bounds__(kRouteThreads) route_count_kernel(PathArgs a, 
 
 // One block: packed-row layout of the buckets and the pair-tile list.
 __global__ void __launch_bounds__(kRouteThreads) route_plan_kernel(PathArgs a, SparseArgs s) {
-  pdl_enter();
   const int nb = a.gp * a.d.E;
   __shared__ int s_rows[kRouteThreads], s_pairs[kRouteThreads];
   // each thread owns a contiguous range of buckets
@@ -168,7 +165,6 @@ __host__ __device__ __forceinline__ int fill_chunk_rows(int rows_max) {
 }
 
 __global__ void __launch_bounds__(kRouteThreads) route_fill_kernel(PathArgs a, SparseArgs s) {
-  pdl_enter();
   const int g = blockIdx.x, m = blockIdx.y, grp = a.g0 + g, E = a.d.E, b = g * E + m;
   if (s.plan[1] == 0) return;
   const int n_rows = n_rows_of(a);
@@ -228,7 +224,6 @@ __global__ void __launch_bounds__(kRouteThreads) route_fill_kernel(PathArgs a, S
 // rows p = x * rpb + t / vpr, stepping by gridDim.x * rpb, thread t the row's
 // vector t % vpr; all index arithmetic per row is a shift or one small division.
 __global__ void __launch_bounds__(256) pack_kernel(PathArgs a, SparseArgs s) {
-  pdl_enter();
   const Dims& d = a.d;
   const int rows = s.plan[1];
   const int vpr = d.d_s / 8;     // 16-byte vectors per head row (<= 256, checked at launch)
@@ -267,7 +262,6 @@ __global__ void __launch_bounds__(256) pack_kernel(PathArgs a, SparseArgs s) {
 // y = sum over the top_k slots (in slot order) -> bf16 target rows.
 // grid (ceil(tpad * D_t / 8 / 256), gp): one thread per 8 channels of a row.
 __global__ void combine_kernel(PathArgs a, SparseArgs s) {
-  pdl_enter();
   const Dims& d = a.d;
   const int g = blockIdx.y, grp = a.g0 + g, K = d.top_k;
   const int vpr = d.Dt / 8;
@@ -306,28 +300,30 @@ cudaError_t launch_route(const PathArgs& a, const SparseArgs& s, int step, cudaS
   if (a.gp <= 0) return cudaSuccess;
   const dim3 grid(a.gp, a.d.E);
   if (step == 0) {
-    return launch_kernel(a.overlap, route_count_kernel, grid, kRouteThreads, 0, st, a, s);
+    route_count_kernel<<<grid, kRouteThreads, 0, st>>>(a, s);
   } else if (step == 1) {
-    return launch_kernel(a.overlap, route_plan_kernel, 1, kRouteThreads, 0, st, a, s);
+    route_plan_kernel<<<1, kRouteThreads, 0, st>>>(a, s);
   } else {
     const int rows_max = a.d.tiles_max * kTileM, chunk = fill_chunk_rows(rows_max);
-    return launch_kernel(a.overlap, route_fill_kernel,
-                         dim3(a.gp, a.d.E, (rows_max + chunk - 1) / chunk), kRouteThreads, 0, st, a, s);
+    route_fill_kernel<<<dim3(a.gp, a.d.E, (rows_max + chunk - 1) / chunk), kRouteThreads, 0, st>>>(a, s);
   }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_pack(const PathArgs& a, const SparseArgs& s, cudaStream_t st) {
   if (a.gp <= 0) return cudaSuccess;
   if (a.d.d_s % 8 || a.d.d_s / 8 > 256 || a.d.H_s <= 0) return cudaErrorInvalidValue;
   const dim3 grid(static_cast<unsigned>(std::max(1, 8 * 152 / a.d.H_s)), a.d.H_s);
-  return launch_kernel(a.overlap, pack_kernel, grid, 256, 0, st, a, s);
+  pack_kernel<<<grid, 256, 0, st>>>(a, s);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_combine(const PathArgs& a, const SparseArgs& s, cudaStream_t st) {
   if (a.gp <= 0) return cudaSuccess;
   const size_t per = static_cast<size_t>(a.d.tpad) * (a.d.Dt / 8);
   const dim3 grid(static_cast<unsigned>((per + 255) / 256), a.gp);
-  return launch_kernel(a.overlap, combine_kernel, grid, 256, 0, st, a, s);
+  combine_kernel<<<grid, 256, 0, st>>>(a, s);
+  return cudaGetLastError();
 }
 
 }  // namespace mot
