@@ -867,7 +867,6 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
 
   const size_t G = bd.G, N = bd.N, D = bd.d, df = bd.df, R = size_t(bd.R), E = bd.E;
   bt.scan = bt_scan_supported(bd) && int64_t(N) * bd.G * bd.B * bd.S <= INT32_MAX / 2;
-  const size_t slots = bt.scan ? N : 1;
   struct A { void** p; size_t n; } allocs[] = {
       {(void**)&bt.prm, bt.scan ? G * N * bt_scan_prm_floats(bd) * 4 : 16},
       {&bt.wg, 2 * E * N * bd.Ds * 2}, {(void**)&bt.bg, 2 * E * 4},
@@ -875,7 +874,7 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
       {(void**)&bt.c_q, G * N * D * 4}, {(void**)&bt.c_kv, G * N * 2 * D * 4},
       {(void**)&bt.c_o, G * N * D * 4}, {(void**)&bt.c_f1, G * N * df * 4},
       {(void**)&bt.c_f2, G * N * D * 4}, {(void**)&bt.c_out, G * bd.Dt * 4},
-      {(void**)&bt.s_out, G * bd.Dt * 4}, {(void**)&bt.rstat, slots * G * R * 8},
+      {(void**)&bt.s_out, G * bd.Dt * 4},
       {(void**)&bt.ln_q, G * N * 2 * D * 4}, {(void**)&bt.ln_c, G * N * 2 * D * 4},
       {(void**)&bt.ln_f, G * N * 2 * D * 4},
       {&bt.win, G * D * 2 * bd.d_s * 2}, {&bt.wq, G * N * D * D * 2}, {&bt.wkv, G * N * 2 * D * D * 2},
@@ -885,7 +884,7 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
       {(void**)&bt.h, G * R * D * 4}, {(void**)&bt.ht, G * R * D * 4},
       {&bt.xz, G * R * D * 2}, {&bt.xq, G * R * D * 2}, {&bt.q, G * R * D * 2},
       {&bt.kv, G * R * 2 * D * 2}, {&bt.o, G * R * D * 2}, {&bt.xf, G * R * D * 2},
-      {&bt.f, df % 128 ? G * R * df * 2 : 16}, {&bt.xo, slots * G * R * D * 2},
+      {&bt.f, df % 128 ? G * R * df * 2 : 16},
       {(void**)&bt.rcnt, 64 * 4}, {(void**)&bt.rlist, G * size_t(bd.B) * bd.S * 4},
       {(void**)&bt.rpre, (2 * G + 2) * 4},
       {&bt.xs, bd.top_k == 1 ? G * R * bd.d_s * 2 : 16},
@@ -893,6 +892,29 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
   for (auto& a : allocs) {
     if (cudaMalloc(a.p, std::max<size_t>(a.n, 16)) != cudaSuccess) {
       cudaGetLastError();
+      free_all(h);
+      delete h;
+      return MOT_ERR_OOM;
+    }
+  }
+  // the scan keeps the state rows of every slot; where they do not fit, those of one slot at
+  // a time and the staged kernels
+  size_t slots = bt.scan ? N : 1;
+  auto state_rows = [&] {
+    if (cudaMalloc((void**)&bt.xo, slots * G * R * D * 2) == cudaSuccess &&
+        cudaMalloc((void**)&bt.rstat, slots * G * R * 8) == cudaSuccess)
+      return true;
+    cudaGetLastError();
+    if (bt.xo) cudaFree(bt.xo);
+    bt.xo = nullptr;
+    bt.rstat = nullptr;
+    return false;
+  };
+  if (!state_rows()) {
+    const bool one_slot = slots > 1;
+    bt.scan = false;
+    slots = 1;
+    if (!one_slot || !state_rows()) {
       free_all(h);
       delete h;
       return MOT_ERR_OOM;

@@ -102,3 +102,32 @@ def test_scan_keeps_non_finite_tokens_apart():
                         assert torch.isnan(y[l, b, :, s].float()).all()
                     else:
                         assert torch.equal(G.int_view(c[l, b, :, s]), G.int_view(x[l, b, :, s]))
+
+
+def test_no_room_for_every_slot_runs_the_staged_kernels():
+    """Where the state rows of all slots (519 MB here) do not fit but those of one slot do
+    (410 MB of workspace in all), the handle is created all the same and a call runs the staged
+    schedule: its launches, and its output bit for bit."""
+    lens = (40, 7)
+    wl = W("bt_room", 1, 16, 64, 16, 2, 32, 2, 0, 2, 1024, "bf16", lens, bt=(0, 16, 128, 4, 128))
+    sk, sv, blob = _inputs(wl, 11)
+    want = _run(wl, sk, sv, blob, staged=True)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    h = M.mot_create_bt(*M.bt_config_from(wl))
+    M.mot_destroy(h)
+    k, v = G.to_device(wl, sk), G.to_device(wl, sv)
+    (_, dk), (_, dv) = G.alloc_dst(wl), G.alloc_dst(wl)
+    lens_d = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    free = torch.cuda.mem_get_info()[0]
+    held = torch.empty(free - (720 << 20), dtype=torch.uint8, device="cuda")
+    h = M.mot_create_bt(*M.bt_config_from(wl))
+    del held
+    torch.cuda.empty_cache()
+    M.mot_load_weights(h, blob)
+    c0 = M.mot_get_launch_count(h)
+    M.mot_translate_bt(h, k, v, lens_d, wl.batch, dk, dv)
+    assert M.mot_get_device_status(h) == M.MOT_OK
+    assert M.mot_get_launch_count(h) - c0 == want[2]
+    assert torch.equal(G.int_view(dk), G.int_view(want[0]))
+    assert torch.equal(G.int_view(dv), G.int_view(want[1]))
