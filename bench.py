@@ -503,9 +503,8 @@ class _Setup:
         if M.mot_get_routing(self.h) == M.ROUTING_SPARSE:
             sched = "routed (Top-K token buckets)"
         if wl.is_bt:
-            sched = ("backbone scan on Top-1 token buckets (8 launches per window slot)"
-                     if M.mot_get_routing(self.h) == 1 else
-                     "backbone scan (7 launches per window slot)")
+            sched = ("backbone scan" + (" on Top-1 token buckets" if M.mot_get_routing(self.h) == 1 else "")
+                     + ", the window in one launch (the kernel list times its stages one by one)")
         self.schedule = sched
         self.bf = wl.dtype == "bf16"
         tdt = torch.bfloat16 if self.bf else torch.float32
@@ -545,7 +544,8 @@ def time_device(M, torch, S, args, world, rank, local):
     sampler = ClockSampler(local) if rank == 0 else None
     if sampler:
         sampler.start()
-    M.mot_profile_enable(S.h, True)
+    # a profiled backbone call runs its stages as separate kernels, so those are timed afterwards
+    M.mot_profile_enable(S.h, not S.wl.is_bt)
     M.mot_profile_read(S.h)
     launches0 = M.mot_get_launch_count(S.h)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -561,9 +561,14 @@ def time_device(M, torch, S, args, world, rank, local):
         dist.barrier()
     elapsed_ms = e0.elapsed_time(e1)
     launches = M.mot_get_launch_count(S.h) - launches0
+    clocks = sampler.stop() if sampler else None
+    if S.wl.is_bt:
+        M.mot_profile_enable(S.h, True)
+        for _ in range(args.steps):
+            S.step()
+        torch.cuda.synchronize()
     kstats = M.mot_profile_read(S.h)
     M.mot_profile_enable(S.h, False)
-    clocks = sampler.stop() if sampler else None
     status = M.mot_get_device_status(S.h, S.stream)
     if status != M.MOT_OK:
         raise SystemExit(f"{S.wl.name}: device status {M.mot_status_string(status)}")
