@@ -441,7 +441,7 @@ mot_status run_translate(mot_ctx* h, const void* src_k, const void* src_v, const
       }));
     } else {
       MOT_CUDA_TRY(timed(h, "simt_gemm1_gelu_gate", st, [&] { return launch_simt_gemm1(a, st); }));
-      MOT_CUDA_TRY(timed(h, "simt_gemm2_combine_store", st, [&] { return launch_simt_gemm2(a, st); }));
+      MOT_CUDA_TRY(timed(h, "simt_gemm2_combine_store", st, [&] { return launch_simt_gemm2(a, h->num_sms, st); }));
     }
   }
   return MOT_OK;

@@ -29,24 +29,37 @@ struct NvtxRange {
 // chain then waits for the one before it, so a chain completes in order. The launch and
 // prologue of a kernel (barriers, tensor-memory allocation, descriptors) hide behind its
 // predecessor's last CTAs, which matters where kernels are short: 57.6 -> 53.0 us for a 64-token
-// mixture of 24 x 128 x 128 blocks, 121 -> 114.7 us for 64 tokens in fp32. Tensor memory is
+// mixture of 24 x 128 x 128 blocks, 121 -> 114.7 us for 64 tokens in fp32 (104.6 since). Tensor memory is
 // allocated before pdl_enter, so no dependent can hold what its predecessor still waits for.
 // Not used by the Top-K passes (their waiting CTAs hold back the pack and combine kernels:
-// 3.41 -> 3.45 ms) nor by the backbone chain (no gain).
+// 3.41 -> 3.45 ms) nor by the backbone chain (no gain). launch_kernel_clusters also groups
+// `cluster_z` CTAs along z into a cluster.
 template <class... P, class... A>
-cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
-                          cudaStream_t st, A&&... args) {
+cudaError_t launch_kernel_clusters(bool overlap, unsigned cluster_z, void (*kernel)(P...), dim3 grid,
+                                   dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchAttribute attr[2] = {};
+  if (overlap) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster_z > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = 1;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = cluster_z;
+  }
+  cfg.attrs = attr;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, A&&... args) {
+  return launch_kernel_clusters(overlap, 1, kernel, grid, block, smem, st, std::forward<A>(args)...);
 }
 
 constexpr int kTileM = 128;   // tokens per token tile (rows of one MMA tile)
@@ -155,7 +168,7 @@ cudaError_t launch_prep(const int32_t* seq_lens, int32_t batch, const Dims& d, T
 cudaError_t launch_gate(const PathArgs& a, cudaStream_t st);
 cudaError_t launch_fixed_gate(const PathArgs& a, const float* fg, cudaStream_t st);
 cudaError_t launch_simt_gemm1(const PathArgs& a, cudaStream_t st);
-cudaError_t launch_simt_gemm2(const PathArgs& a, cudaStream_t st);
+cudaError_t launch_simt_gemm2(const PathArgs& a, int num_sms, cudaStream_t st);
 
 // tcgen05 path. GEMM1: source K/V load maps, W1 load map and the A2 store map
 // (box 64 x 32 x 1); GEMM2: A2 load map (box 64 x 128 x 1) and W2 load map.

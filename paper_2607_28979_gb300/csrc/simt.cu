@@ -15,11 +15,11 @@
 // at the end. Three K blocks are in flight (cp.async for fp32 rows).
 //
 // What bounds it: one 64-token context (4 layers, E = 2, 768-768-768) is 2.42 GFLOP, 32 us
-// at 128 FMA per SM and clock, on 384 and 192 CTAs; the 16-byte reads take the load path for
-// 1.5 times the FMAs' cycles, and the second GEMM's CTAs fill 1.3 waves. Measured there: 160
+// at 128 FMA per SM and clock, on 384 CTAs each (the second GEMM's 192 tiles split over pairs);
+// the 16-byte reads take the load path for 1.5 times the FMAs' cycles. Measured there: 160
 // and 209 us as 64 x 64 tiles of 4 x 4 threads (two scalar-fed reads per 16 FMAs, half of the
-// SMs idle), 49 and 59 us so; 8 x 8 outputs a thread take 55 and 67 us with packed pairs (one
-// CTA per SM) and 54 and 58 us with single FMAs.
+// SMs idle), 49 and 59 us as 64 x 32 tiles, 49 and 50 us with the pairs; 8 x 8 outputs a thread
+// took 55 and 67 us with packed pairs (one CTA per SM) and 54 and 58 us with single FMAs.
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -68,10 +68,18 @@ __device__ __forceinline__ void ld_pairs(uint32_t addr, uint64_t& a, uint64_t& b
   asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
 }
 
-// GEMM 1 or 2. Grid (2 * tiles_max, columns / 32, gp): blockIdx.x is a 64-row half tile.
+__device__ __forceinline__ float ld_peer(uint32_t addr) {   // another CTA's shared memory
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+// GEMM 1 or 2. Grid (2 * tiles_max, columns / 32, gp * KS): blockIdx.x is a 64-row half tile.
 // VEC: d_s and both K lengths are multiples of four, so every four-value piece is aligned and
-// inside one row and head; otherwise values are read one by one.
-template <typename T, int GEMM, bool VEC>
+// inside one row and head; otherwise values are read one by one. KS = 2 (GEMM2): a cluster of two
+// CTAs, each with half of the K blocks; each then sums and stores half of the tile's rows, reading
+// the other's partial sums from its shared memory.
+template <typename T, int GEMM, bool VEC, int KS>
 __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathArgs a) {
   using TA = typename std::conditional<GEMM == 1, T, float>::type;   // the A operand's type
   extern __shared__ float4 simt_smem4[];
@@ -83,7 +91,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
   const TileInfo ti = a.tiles[m];
   const int row0 = (blockIdx.x & 1) * BM;   // row offset inside the 128-row tile
   if (row0 >= ti.rows) return;
-  const int gl = blockIdx.z, grp = a.g0 + gl;
+  const int gl = blockIdx.z / KS, half = blockIdx.z % KS, grp = a.g0 + gl;
   const GroupInfo gi = a.groups[grp];
   const int n0 = blockIdx.y * BN;
   const int K = GEMM == 1 ? d.Ds : d.EH, N = GEMM == 1 ? d.EH : d.Dt;
@@ -167,13 +175,14 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
     for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
   const uint32_t sbase = smem_u32(sm);
   const uint32_t aoff = (ty * kLd + kg * 16) * 4, boff = ((BM + tx) * kLd + kg * 16) * 4;
-  const int nk = (K + BK - 1) / BK;
+  const int nk_all = (K + BK - 1) / BK, per = (nk_all + KS - 1) / KS;
+  const int k0 = half * per, nk = min(nk_all, k0 + per);
 #pragma unroll
   for (int s = 0; s < kSimtStages - 1; ++s) {
-    if (s < nk) load(s);
+    if (k0 + s < nk) load(k0 + s);
     else cp_async_commit();
   }
-  for (int kb = 0; kb < nk; ++kb) {
+  for (int kb = k0; kb < nk; ++kb) {
     cp_async_wait_group<kSimtStages - 2>();
     __syncthreads();   // block kb landed; every thread is done with block kb - 1
     if (kb + kSimtStages - 1 < nk) load(kb + kSimtStages - 1);
@@ -206,14 +215,24 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
       sm[(kg * BM + ty + 8 * i) * BN + tx + 8 * j] =
           __uint_as_float(static_cast<uint32_t>(acc[i][j])) +
           __uint_as_float(static_cast<uint32_t>(acc[i][j] >> 32));
-  __syncthreads();
+  if (KS > 1) cluster_sync();
+  else __syncthreads();
   const int col = n0 + (tid & 31);   // a warp takes a row's 32 columns
-  if (col >= N) return;
-  for (int r = tid >> 5; r < nrows; r += kSimtThreads / 32) {
-    const float* p = sm + r * BN + (tid & 31);
-    float y = p[0];
+  const int r0 = (tid >> 5) + half * (kSimtThreads / 32);
+  const uint32_t peer = KS > 1 ? mapa_cluster(sm, 1 - half) : 0;
+  for (int r = r0; r < nrows && col < N; r += KS * kSimtThreads / 32) {
+    const int o = r * BN + (tid & 31);
+    float y = sm[o];
 #pragma unroll
-    for (int k = 1; k < kKGroups; ++k) y += p[k * BM * BN];
+    for (int k = 1; k < kKGroups; ++k) y += sm[o + k * BM * BN];
+    if (KS > 1) {
+      float z[kKGroups];
+#pragma unroll
+      for (int k = 0; k < kKGroups; ++k) z[k] = ld_peer(peer + (o + k * BM * BN) * 4);
+#pragma unroll
+      for (int k = 1; k < kKGroups; ++k) z[0] += z[k];
+      y += z[0];
+    }
     const size_t grow = static_cast<size_t>(m) * kTileM + row0 + r;
     const float* g = a.gate + (static_cast<size_t>(grp) * d.tpad + grow) * d.E;
     if (GEMM == 1) {
@@ -230,37 +249,58 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
            y);
     }
   }
+  if (KS > 1) {   // the other CTA may still read this one's sums
+    __syncwarp();
+    cluster_sync();
+  }
 }
 
-template <typename T, int GEMM, bool VEC>
+template <typename T, int GEMM, bool VEC, int KS>
 cudaError_t launch_simt_v(const PathArgs& a, cudaStream_t st) {
   const Dims& d = a.d;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(simt_gemm_kernel<T, GEMM, VEC>,
+    cudaError_t e = cudaFuncSetAttribute(simt_gemm_kernel<T, GEMM, VEC, KS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kSimtSmem);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const int N = GEMM == 1 ? d.EH : d.Dt;
-  dim3 grid(2 * d.tiles_max, (N + BN - 1) / BN, a.gp);
-  return launch_kernel(a.overlap, simt_gemm_kernel<T, GEMM, VEC>, grid, kSimtThreads, kSimtSmem, st, a);
+  dim3 grid(2 * d.tiles_max, (N + BN - 1) / BN, a.gp * KS);
+  return launch_kernel_clusters(a.overlap, KS, simt_gemm_kernel<T, GEMM, VEC, KS>, grid, kSimtThreads,
+                                kSimtSmem, st, a);
 }
 
-template <typename T, int GEMM>
+template <typename T, int GEMM, int KS>
 cudaError_t launch_simt(const PathArgs& a, cudaStream_t st) {
-  return a.d.d_s % 4 == 0 && a.d.EH % 4 == 0 ? launch_simt_v<T, GEMM, true>(a, st)
-                                             : launch_simt_v<T, GEMM, false>(a, st);
+  return a.d.d_s % 4 == 0 && a.d.EH % 4 == 0 ? launch_simt_v<T, GEMM, true, KS>(a, st)
+                                             : launch_simt_v<T, GEMM, false, KS>(a, st);
+}
+
+// GEMM2's K split over a pair: where the tiles fill the SMs' two places each at most once, and
+// up to eight times over when K is long enough for the exchange not to count. E * H = 1536, 64
+// tokens (192 tiles): 59.9 -> 49.6 us; 6144: 202 -> 154 us; 200 tokens (768 tiles): 557 -> 512
+// us; 512 tokens: 1,021 -> 978 us; K = 768: 35.2 -> 32.2 us. Beyond: 1,751 -> 1,757 us (600 +
+// 300 tokens, 6144), 110 -> 115 us (3 x 64 tokens, 1536), 26.8 -> 26.6 us (K = 512), 19.3 ->
+// 20.5 us (K = 256).
+template <typename T>
+cudaError_t launch_simt2(const PathArgs& a, int num_sms, cudaStream_t st) {
+  const Dims& d = a.d;
+  const long long tiles = static_cast<long long>(d.B) * ((d.S + BM - 1) / BM) *
+                          ((d.Dt + BN - 1) / BN) * a.gp;
+  const bool split = d.EH >= 8 * BK && (tiles <= 2ll * num_sms ||
+                                        (d.EH >= 64 * BK && tiles <= 16ll * num_sms));
+  return split ? launch_simt<T, 2, 2>(a, st) : launch_simt<T, 2, 1>(a, st);
 }
 
 }  // namespace
 
 cudaError_t launch_simt_gemm1(const PathArgs& a, cudaStream_t st) {
-  return a.d.dtype == 0 ? launch_simt<__nv_bfloat16, 1>(a, st) : launch_simt<float, 1>(a, st);
+  return a.d.dtype == 0 ? launch_simt<__nv_bfloat16, 1, 1>(a, st) : launch_simt<float, 1, 1>(a, st);
 }
 
-cudaError_t launch_simt_gemm2(const PathArgs& a, cudaStream_t st) {
-  return a.d.dtype == 0 ? launch_simt<__nv_bfloat16, 2>(a, st) : launch_simt<float, 2>(a, st);
+cudaError_t launch_simt_gemm2(const PathArgs& a, int num_sms, cudaStream_t st) {
+  return a.d.dtype == 0 ? launch_simt2<__nv_bfloat16>(a, num_sms, st) : launch_simt2<float>(a, num_sms, st);
 }
 
 }  // namespace mot
