@@ -337,38 +337,69 @@ __device__ void epi_plain(const EpiCtx& e, const Work& w, uint32_t tb, int row, 
   }
 }
 
+// A row's 32 output channels (64 bytes) at `o`: whole 32-byte sectors where `wide` (o 32-byte
+// aligned), else 16-byte pieces.
+__device__ __forceinline__ void store_out_row(uint16_t* o, const float (&y)[32], bool wide) {
+  uint32_t p[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) p[k] = pack2(y[2 * k], y[2 * k + 1]);
+  if (wide) {
+    st_global_v8(o, p);
+    st_global_v8(o + 16, p + 8);
+  } else {
+    uint4* o4 = reinterpret_cast<uint4*>(o);
+#pragma unroll
+    for (int q8 = 0; q8 < 4; ++q8)
+      o4[q8] = make_uint4(p[4 * q8], p[4 * q8 + 1], p[4 * q8 + 2], p[4 * q8 + 3]);
+  }
+}
+
 // kBtOut: the E backbones' accumulators of this 128-token tile sit side by
 // side (E * NT columns); the gate-weighted sum goes to target layer q0 + r.
 // Routed (Top-1): one bucket's accumulator for 128 of its positions; each row
 // is its token's whole output (gtilde = 1), stored at the token's position.
-__device__ void epi_out_routed(const EpiCtx& e, const Work& w, uint32_t tb, int row, int cg,
+// What bounds it: the epilogue, whose rows go to scattered places. 4 x 4096 slots (7,923 tokens)
+// of 2 heads, 8 slots of 256 outputs: 62 us with 16-byte stores and every row's values read
+// after its accumulators were complete, 59 us with those made by the idle warps a tile ahead and
+// the vectors in 16-byte reads, 44 us with 32-byte stores (whole sectors).
+//
+// What a row needs besides its accumulators, made by warps 2 and 3 while the epilogue works on
+// the tile before: its position in the target (layer rows of head 0; negative: no row), the gate
+// weight, and LN_out's mean and reciprocal deviation over the token's P rows (Chan's combination
+// of the per-row mean and M2, each over d values).
+__device__ float4 out_row(const BtArgs& a, const Work& w, int row) {
+  const BtDims& d = a.d;
+  const int g = w.g, x = g / d.E, m = g - x * d.E;
+  if (row >= w.ntok) return make_float4(__int_as_float(-1), 0.f, 0.f, 0.f);
+  const int pos = w.tok0 + row;
+  const int tok = a.list[int64_t(g) * d.B * d.S + pos];
+  const float2* st = a.rstat + (int64_t(w.r) * d.G + g) * d.R + int64_t(pos) * d.P;
+  const float gt = a.gate[(int64_t(x) * d.B * d.S + tok) * d.E + m];
+  float tm = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < d.P; ++k) tm += st[k].x;
+  tm /= d.P;
+  float tq = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < d.P; ++k) {
+    const float2 sk = st[k];
+    tq += sk.y + d.d * (sk.x - tm) * (sk.x - tm);
+  }
+  return make_float4(__int_as_float(tok), gt, tm, rsqrtf(tq / (float(d.d) * d.P) + kLnEps));
+}
+
+__device__ void epi_out_routed(const EpiCtx& e, const Work& w, uint32_t tb, float4 rw, int cg,
                                int ng) {
   const BtArgs& a = *e.a;
   const GemmCfg& c = *e.c;
   const BtDims& d = a.d;
-  const int g = w.g, x = g / d.E, m = g - x * d.E;
-  const int pos = w.tok0 + row;
-  const bool valid = row < w.ntok;
-  int b = 0, s = 0;
-  float gt = 0.f, mu = 0.f, rs = 0.f;
-  if (valid) {
-    const int tok = a.list[int64_t(g) * d.B * d.S + pos];
-    b = tok / d.S;
-    s = tok - b * d.S;
-    gt = a.gate[(int64_t(x) * d.B * d.S + tok) * d.E + m];
-    const float2* st = a.rstat + (int64_t(w.r) * d.G + g) * d.R + int64_t(pos) * d.P;
-    float tm = 0.f;
-    for (int k = 0; k < d.P; ++k) tm += st[k].x;
-    tm /= d.P;
-    float tq = 0.f;
-    for (int k = 0; k < d.P; ++k) {
-      const float2 sk = st[k];
-      tq += sk.y + d.d * (sk.x - tm) * (sk.x - tm);
-    }
-    mu = tm;
-    rs = rsqrtf(tq / (float(d.d) * d.P) + kLnEps);
-  }
+  const int g = w.g, x = g / d.E;
+  const int tok = __float_as_int(rw.x);
+  const bool valid = tok >= 0;
+  const int b = tok / d.S, s = tok - b * d.S;
+  const float gt = rw.y, mu = rw.z, rs = rw.w;
   uint16_t* dst = static_cast<uint16_t*>(a.dst[x]);
+  const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31u) == 0;   // d_t is a multiple of 32
   const int l = d.q0 + a.slot + w.r;
   const float* cbase = a.c_out + int64_t(g) * d.Dt;
   const float* sbase = a.s_out + int64_t(g) * d.Dt;
@@ -378,21 +409,20 @@ __device__ void epi_out_routed(const EpiCtx& e, const Work& w, uint32_t tb, int 
     tmem_ld_32x32b_x32(tb + ch * 32, rr);
     tmem_ld_wait(rr);
     if (!valid) continue;
-    const int col = w.j * c.NT + ch * 32;
+    const int col = w.j * c.NT + ch * 32;   // D_t is a multiple of 32, so the vectors are aligned
+    const float4* s4 = reinterpret_cast<const float4*>(sbase + col);
+    const float4* c4 = reinterpret_cast<const float4*>(cbase + col);
     float y[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const float u = fmaf(__uint_as_float(rr[k]) - mu * __ldg(sbase + col + k), rs,
-                           __ldg(cbase + col + k));
-      y[k] = fmaf(gt, gelu_tanh(u), 0.f);
+    for (int k = 0; k < 32; k += 4) {
+      const float4 sv = __ldg(s4 + k / 4), cv = __ldg(c4 + k / 4);
+      y[k] = fmaf(gt, gelu_tanh(fmaf(__uint_as_float(rr[k]) - mu * sv.x, rs, cv.x)), 0.f);
+      y[k + 1] = fmaf(gt, gelu_tanh(fmaf(__uint_as_float(rr[k + 1]) - mu * sv.y, rs, cv.y)), 0.f);
+      y[k + 2] = fmaf(gt, gelu_tanh(fmaf(__uint_as_float(rr[k + 2]) - mu * sv.z, rs, cv.z)), 0.f);
+      y[k + 3] = fmaf(gt, gelu_tanh(fmaf(__uint_as_float(rr[k + 3]) - mu * sv.w, rs, cv.w)), 0.f);
     }
     const int hh = col / d.d_t, i0 = col - hh * d.d_t;
-    uint4* o4 = reinterpret_cast<uint4*>(
-        dst + (((int64_t(l) * d.B + b) * d.H_t + hh) * d.S + s) * d.d_t + i0);
-#pragma unroll
-    for (int q8 = 0; q8 < 4; ++q8)
-      o4[q8] = make_uint4(pack2(y[8 * q8], y[8 * q8 + 1]), pack2(y[8 * q8 + 2], y[8 * q8 + 3]),
-                          pack2(y[8 * q8 + 4], y[8 * q8 + 5]), pack2(y[8 * q8 + 6], y[8 * q8 + 7]));
+    store_out_row(dst + (((int64_t(l) * d.B + b) * d.H_t + hh) * d.S + s) * d.d_t + i0, y, wide);
   }
 }
 
@@ -425,6 +455,7 @@ __device__ void epi_out(const EpiCtx& e, const Work& w, uint32_t tb, int row, in
     rs[m] = rsqrtf(tq / (float(d.d) * d.P) + kLnEps);
   }
   uint16_t* dst = static_cast<uint16_t*>(a.dst[x]);
+  const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31u) == 0;   // d_t is a multiple of 32
   const int l = d.q0 + a.slot + w.r;
   for (int ch = cg; ch < c.NT / 32; ch += ng) {
     float y[32];
@@ -447,12 +478,7 @@ __device__ void epi_out(const EpiCtx& e, const Work& w, uint32_t tb, int row, in
     }
     if (!valid) continue;
     const int hh = col / d.d_t, i0 = col - hh * d.d_t;
-    uint4* o4 = reinterpret_cast<uint4*>(
-        dst + (((int64_t(l) * d.B + b) * d.H_t + hh) * d.S + s) * d.d_t + i0);
-#pragma unroll
-    for (int q8 = 0; q8 < 4; ++q8)
-      o4[q8] = make_uint4(pack2(y[8 * q8], y[8 * q8 + 1]), pack2(y[8 * q8 + 2], y[8 * q8 + 3]),
-                          pack2(y[8 * q8 + 4], y[8 * q8 + 5]), pack2(y[8 * q8 + 6], y[8 * q8 + 7]));
+    store_out_row(dst + (((int64_t(l) * d.B + b) * d.H_t + hh) * d.S + s) * d.d_t + i0, y, wide);
   }
 }
 
@@ -472,9 +498,11 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
   uint64_t* tfull = empty + kBtStages;   // [2]
   uint64_t* tempty = tfull + 2;          // [2]
   uint64_t* drain = tempty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  uint64_t* rfull = drain + 1;           // [2] routed output: the rows' values are in place
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rfull + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float2* xch = reinterpret_cast<float2*>(smem + kBtStages * kBtStageBytes + 256);   // [2][2][128]
+  float4* orow = reinterpret_cast<float4*>(xch);   // [2][128] (the row-norm stages alone use xch)
 
   const BtDims& d = a.d;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -491,6 +519,7 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], EPI);
+      mbar_init(&rfull[b], 2);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -599,7 +628,30 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
       buf ^= 1;
       if (buf == 0) buf_phase ^= 1u;
     }
-  } else if (warp >= 4) {
+  } else if (warp < 4) {
+    // ------------------------------------------------ routed output: each row's values, 64 rows a warp
+    if (EPI == 16 && is_out && a.routed) {
+      int buf = 0;
+      uint32_t buf_phase = 0;
+      for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        const Work w = decode(a, c, it);
+        if (!w.active) continue;
+        float4 v[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) v[i] = out_row(a, w, (warp - 2) * 64 + i * 32 + lane);
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait(&tempty[buf], buf_phase ^ 1u, abort_flag, a.wait_limit) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) orow[buf * 128 + (warp - 2) * 64 + i * 32 + lane] = v[i];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&rfull[buf]);
+        buf ^= 1;
+        if (buf == 0) buf_phase ^= 1u;
+      }
+    }
+  } else {
     // ------------------------------------------------ epilogue
     const int q = warp & 3;
     const int cg = (warp - 4) >> 2;   // column group of this warp (EPI / 4 groups)
@@ -611,11 +663,16 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
       const Work w = decode(a, c, it);
       if (!w.active) continue;
       int ok = 1;
-      if (lane == 0) ok = mbar_wait(&tfull[buf], buf_phase, abort_flag, a.wait_limit) ? 1 : 0;
+      if (lane == 0) {
+        ok = mbar_wait(&tfull[buf], buf_phase, abort_flag, a.wait_limit) ? 1 : 0;
+        if (EPI == 16 && is_out && a.routed && ok)
+          ok = mbar_wait(&rfull[buf], buf_phase, abort_flag, a.wait_limit) ? 1 : 0;
+      }
       ok = __shfl_sync(0xffffffffu, ok, 0);
       // the split rows pair warps at a barrier: every epilogue warp stops, or none
       if constexpr (EPI == kBtRowEpi) ok = epi_and(1, 32 * EPI, ok != 0) ? 1 : 0;
       if (!ok) break;
+      __syncwarp();   // orow, behind lane 0's wait
       tc_fence_after();
       const uint32_t tb = tmem_base + static_cast<uint32_t>(buf * acc_cols) +
                           (static_cast<uint32_t>(q * 32) << 16);
@@ -623,7 +680,7 @@ __global__ void __launch_bounds__(bt_threads(EPI), 1)
         epi_row<D, 2>(e, w, tb, row, RowXch{xch + buf * 256, cg, 32 * EPI});
       } else {
         if (c.mode == kBtOut && a.routed)
-          epi_out_routed(e, w, tb, row, cg, EPI / 4);
+          epi_out_routed(e, w, tb, orow[buf * 128 + row], cg, EPI / 4);
         else if (c.mode == kBtOut)
           epi_out(e, w, tb, row, cg, EPI / 4);
         else

@@ -124,11 +124,7 @@ __device__ __forceinline__ void store_out32(const uint32_t (&acc)[32], __nv_bflo
   for (int i = 0; i < 16; ++i)
     w[i] = pack_bf16x2(__uint_as_float(acc[2 * i]), __uint_as_float(acc[2 * i + 1]));
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o + 16 * h),
-                 "r"(w[8 * h]), "r"(w[8 * h + 1]), "r"(w[8 * h + 2]), "r"(w[8 * h + 3]),
-                 "r"(w[8 * h + 4]), "r"(w[8 * h + 5]), "r"(w[8 * h + 6]), "r"(w[8 * h + 7])
-                 : "memory");
+  for (int h = 0; h < 2; ++h) st_global_v8(o + 16 * h, w + 8 * h);
 }
 
 __device__ __forceinline__ void store_out(const uint32_t (&acc)[32], __nv_bfloat16* o) {

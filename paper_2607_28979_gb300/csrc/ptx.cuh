@@ -105,6 +105,13 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// 32 bytes (eight 32-bit words) to a 32-byte-aligned global address.
+__device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* p) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(p[0]),
+               "r"(p[1]), "r"(p[2]), "r"(p[3]), "r"(p[4]), "r"(p[5]), "r"(p[6]), "r"(p[7])
+               : "memory");
+}
+
 // ---------------------------------------------------------------- dependent launches
 //
 // pdl_enter: let the next kernel of the stream start its prologue as SMs come free, and wait

@@ -131,3 +131,26 @@ def test_no_room_for_every_slot_runs_the_staged_kernels():
     assert M.mot_get_launch_count(h) - c0 == want[2]
     assert torch.equal(G.int_view(dk), G.int_view(want[0]))
     assert torch.equal(G.int_view(dv), G.int_view(want[1]))
+
+
+@pytest.mark.parametrize("top_k", [0, 1])
+@pytest.mark.parametrize("staged", [False, True])
+def test_output_rows_at_either_alignment(top_k, staged):
+    """Targets that start 16 bytes past a 32-byte boundary get the same bits (16-byte stores),
+    and nothing around them is written."""
+    wl = W("bt_lead", 2, 3, 64, 3, 3, 32, 2, 0, 2, 70, "bf16", (70, 33), top_k=top_k, bt=(0, 2, 128, 4, 128))
+    sk, sv, blob = _inputs(wl, 13)
+    want = _run(wl, sk, sv, blob, staged)
+    h = M.mot_create_bt(*M.bt_config_from(wl))
+    M.mot_load_weights(h, blob)
+    M.mot_profile_enable(h, staged)
+    k, v = G.to_device(wl, sk), G.to_device(wl, sv)
+    (bk, dk), (bv, dv) = G.alloc_dst(wl, 8), G.alloc_dst(wl, 8)
+    assert dk.data_ptr() % 32 == 16 and want[0].data_ptr() % 32 == 0
+    lens = torch.tensor(wl.seq_lens, dtype=torch.int32, device="cuda")
+    M.mot_translate_bt(h, k, v, lens, wl.batch, dk, dv)
+    assert M.mot_get_device_status(h) == M.MOT_OK
+    for buf, got, ref in ((bk, dk, want[0]), (bv, dv, want[1])):
+        assert torch.equal(G.int_view(got), G.int_view(ref))
+        s = G.sentinel_value(wl)
+        assert bool((G.int_view(buf[:8]) == s).all()) and bool((G.int_view(buf[8 + got.numel():]) == s).all())
