@@ -65,6 +65,7 @@ __device__ __forceinline__ void epilogue_gemm2_sparse(const PathArgs& p, const S
   const bool valid = r < rows_own;
   float* out = nullptr;              // top_k > 1: the token's slot row (fp32)
   __nv_bfloat16* tgt = nullptr;      // top_k = 1: the target cache row, head 0
+  bool wide = false;
   if (valid) {
     const int tok = sp.ltok[p_own + r], slot = sp.lslot[p_own + r];
     if (d.top_k == 1) {
@@ -73,6 +74,7 @@ __device__ __forceinline__ void epilogue_gemm2_sparse(const PathArgs& p, const S
       tgt = static_cast<__nv_bfloat16*>(p.dst[gi.x]) +
             ((static_cast<size_t>(gi.tgt_layer) * d.B + ti.b) * d.H_t * d.S + ti.s0 + tok % UM) *
                 d.d_t;
+      wide = (reinterpret_cast<uintptr_t>(tgt) & 31u) == 0;
     } else {
       out = sp.ybuf + ((static_cast<size_t>(gl) * d.tpad + tok) * d.top_k + slot) * d.Dt + n0;
     }
@@ -84,19 +86,10 @@ __device__ __forceinline__ void epilogue_gemm2_sparse(const PathArgs& p, const S
     tmem_ld_wait(v);
     if (valid && tgt) {   // channel c of head c / d_t, d_t a multiple of 32
       const int c = n0 + ch * 32, h = c / d.d_t, i0 = c - h * d.d_t;
-      uint4* o4 = reinterpret_cast<uint4*>(tgt + static_cast<size_t>(h) * d.S * d.d_t + i0);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        o4[j] = make_uint4(pack_bf16x2(__uint_as_float(v[8 * j + 0]), __uint_as_float(v[8 * j + 1])),
-                           pack_bf16x2(__uint_as_float(v[8 * j + 2]), __uint_as_float(v[8 * j + 3])),
-                           pack_bf16x2(__uint_as_float(v[8 * j + 4]), __uint_as_float(v[8 * j + 5])),
-                           pack_bf16x2(__uint_as_float(v[8 * j + 6]), __uint_as_float(v[8 * j + 7])));
+      store_row32(v, tgt + static_cast<size_t>(h) * d.S * d.d_t + i0, wide);
     } else if (valid) {
-      float4* o4 = reinterpret_cast<float4*>(out + ch * 32);
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        o4[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                            __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+      for (int j = 0; j < 4; ++j) st_global_v8(out + ch * 32 + 8 * j, v + 8 * j);
     }
   }
 }
@@ -124,6 +117,7 @@ __device__ __forceinline__ void epilogue_proj(const PathArgs& p, uint32_t tbase,
   __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.dst[x]);
   const size_t s = static_cast<size_t>(ti.s0) + row;
   const size_t lbase = (static_cast<size_t>(p.proj_layer[grp]) * d.B + ti.b) * d.H_t;
+  const bool wide = (reinterpret_cast<uintptr_t>(dst) & 31u) == 0;   // d_t is a multiple of 32
 #pragma unroll 1
   for (int ch = 0; ch < UN / 32; ++ch) {
     uint32_t r[32];
@@ -131,13 +125,7 @@ __device__ __forceinline__ void epilogue_proj(const PathArgs& p, uint32_t tbase,
     tmem_ld_wait(r);
     if (valid) {
       const int c = c0 + ch * 32, h = c / d.d_t, i0 = c - h * d.d_t;
-      uint4* o4 = reinterpret_cast<uint4*>(dst + ((lbase + h) * d.S + s) * d.d_t + i0);
-#pragma unroll
-      for (int v = 0; v < 4; ++v)
-        o4[v] = make_uint4(pack_bf16x2(__uint_as_float(r[8 * v + 0]), __uint_as_float(r[8 * v + 1])),
-                           pack_bf16x2(__uint_as_float(r[8 * v + 2]), __uint_as_float(r[8 * v + 3])),
-                           pack_bf16x2(__uint_as_float(r[8 * v + 4]), __uint_as_float(r[8 * v + 5])),
-                           pack_bf16x2(__uint_as_float(r[8 * v + 6]), __uint_as_float(r[8 * v + 7])));
+      store_row32(r, dst + ((lbase + h) * d.S + s) * d.d_t + i0, wide);
     }
   }
 }
