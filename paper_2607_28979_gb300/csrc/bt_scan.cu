@@ -28,8 +28,9 @@
 // tensor cores work 7,000). The stages one by one move about 2.2 KB per row and slot through
 // memory in 8 launches a slot; here a slot reads its 128-byte source rows and writes its
 // 256-byte state rows. 8 x 1024 tokens of 12 heads, Top-1 of 2, 4 slots: 2,778 us for the
-// translation staged, 1,098 us with this kernel; 7,923 ragged tokens of 2 heads, 8 slots:
-// 1,362 and 495 us. Steps on the first of these: 16 warps of 32 columns with the vectors read
+// translation staged, 1,098 us with this kernel (987 with the gate, route and projection as they
+// are now); 7,923 ragged tokens of 2 heads, 8 slots:
+// 1,362 and 495 us (375). Steps on the first of these: 16 warps of 32 columns with the vectors read
 // from global memory 1,520 (what L1 the shared memory leaves holds neither them nor spilled
 // registers), vectors staged by the producer and packed fp32 pairs 1,344, attention without
 // integer divisions 1,206, 8 warps of 64 columns 1,214, q ahead of z, v committed apart, the

@@ -126,8 +126,10 @@ __device__ __forceinline__ void epilogue_gemm1(const PathArgs& p, const CUtensor
 
 // 32 fp32 accumulator columns -> 32 bf16 channels at `o`: whole 32-byte sectors where `wide`
 // (o 32-byte aligned), else 16-byte pieces. A warp's rows lie apart, so a 16-byte piece is half a
-// sector: Top-2 GEMM2's fp32 rows 895 -> 798 us (9 layers, 16,384 tokens, D_t = 512), a
-// dense call of 61,440 tokens 42.9 -> 41.6 ms under the power cap.
+// sector. Top-2 GEMM2's fp32 rows: 895 -> 798 us (9 layers, 16,384 tokens, D_t = 512). Dense
+// calls, six runs a side in turn, under the power cap: 16,384 tokens of MoT-h 6.48 -> 6.38 ms,
+// 8 x 1024 of GPT-2-small widths 2.544 -> 2.526 ms, 61,440 of the 7B pair 41.56 -> 41.26 ms (single
+// runs differ by 0.8%).
 __device__ __forceinline__ void store_row32(const uint32_t (&r)[32], __nv_bfloat16* o, bool wide) {
   uint32_t w[16];
 #pragma unroll
