@@ -475,18 +475,25 @@ __global__ void __launch_bounds__(Fa<D>::kThreads, 1)
         tmem_ld_wait(o);
       }
       if (qq < L) {
-        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(a.out) +
-                                              ((int64_t(b) * d.Hq + h) * d.N + qq) * D + c4 * OC);
+        uint16_t* dst = static_cast<uint16_t*>(a.out) +
+                        ((int64_t(b) * d.Hq + h) * d.N + qq) * D + c4 * OC;
+        uint32_t w[OC / 2];
 #pragma unroll
-        for (int e8 = 0; e8 < OC / 8; ++e8) {
-          uint32_t w4[4];
+        for (int e = 0; e < OC / 2; ++e) {
+          __nv_bfloat162 u = __floats2bfloat162_rn(__uint_as_float(o[2 * e]) * inv,
+                                                   __uint_as_float(o[2 * e + 1]) * inv);
+          w[e] = *reinterpret_cast<uint32_t*>(&u);
+        }
+        // whole 32-byte sectors where the output starts on one: 225.5 us a layer of 4 x 4096
+        // positions and 12 heads of 128, 230.4 in 16-byte pieces (half sectors, rows apart)
+        if ((reinterpret_cast<uintptr_t>(a.out) & 31u) == 0) {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            __nv_bfloat162 u = __floats2bfloat162_rn(__uint_as_float(o[8 * e8 + 2 * e]) * inv,
-                                                     __uint_as_float(o[8 * e8 + 2 * e + 1]) * inv);
-            w4[e] = *reinterpret_cast<uint32_t*>(&u);
-          }
-          dst[e8] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+          for (int e = 0; e < OC / 16; ++e) st_global_v8(dst + 16 * e, w + 8 * e);
+        } else {
+#pragma unroll
+          for (int e = 0; e < OC / 8; ++e)
+            reinterpret_cast<uint4*>(dst)[e] =
+                make_uint4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
         }
       }
     }

@@ -47,3 +47,21 @@ def test_target_16_bytes_past_a_sector(name):
         outs.append((G.int_view(dk).clone(), G.int_view(dv).clone()))
     assert all(torch.equal(a, b) for a, b in zip(*outs))
     assert bool((outs[0][0] != G.sentinel_value(wl)).any())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_full_replay_output_16_bytes_past_a_sector(d):
+    wl = synth.ReplayWorkload("al_full", 2, 2, 6, 2, d, 2, 264, (264, 131), top_s=16, n_full=2)
+    h = M.mot_create_replay(M.replay_config_from(wl))
+    q, k, v = (torch.from_numpy(x.view("int16")).cuda() for x in synth.gen_replay_qkv(wl, 5))
+    lens = torch.tensor(wl.seq_lens, dtype=torch.int32, device="cuda")
+    outs = []
+    for lead in (0, 8):
+        n = wl.max_batch * wl.q_heads * wl.max_seq * d
+        buf = torch.full((lead + n + 64,), G.SENTINEL_BF16, dtype=torch.int16, device="cuda")
+        assert buf[lead:].data_ptr() % 32 == 2 * lead
+        M.mot_replay_attention(h, 1, q, k, v, None, lens, len(wl.seq_lens), buf[lead:])
+        torch.cuda.synchronize()
+        assert bool((buf[:lead] == G.SENTINEL_BF16).all()) and bool((buf[lead + n:] == G.SENTINEL_BF16).all())
+        outs.append(buf[lead:lead + n].clone())
+    assert torch.equal(*outs) and bool((outs[0] != G.SENTINEL_BF16).any())
