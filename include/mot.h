@@ -215,7 +215,7 @@ mot_status mot_get_schedule(mot_handle h, int32_t* schedule);
  * name, in first-launch order) and clears the collected events. Backbone
  * handles whose shapes run the window's scan in one launch run its stages one
  * by one while profiling is enabled, so that each has a time of its own; the
- * results agree within the bf16 tolerance.
+ * results agree bit for bit.
  */
 typedef struct {
   char name[32];

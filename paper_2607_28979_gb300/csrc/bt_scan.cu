@@ -5,39 +5,40 @@
 // One persistent CTA per SM walks (group, row tile) items; a tile holds whole tokens (tau x P
 // of its 128 rows). Per slot, as in bt.cu: z = GELU(W_in LN_in(x) + b_in), q from LN_Q(h),
 // k | v from LN_C(z), attention over the token's P rows, h += W_O o + b_O, h += FFN(LN_F(h)).
-// The fp32 state lives in 128 columns of tensor memory for the whole scan: W_O and W_F2
-// accumulate onto it, and the biases they leave out are added, summed over the slots so far,
-// wherever h is read. Rows between the products are bf16 tiles in shared
-// memory, rounded where the staged kernels round them.
+// The fp32 state lives in 128 columns of tensor memory for the whole scan; the residual sums, the
+// layer norms and the attention are fp32 in the order of the staged kernels, and rows between the
+// products are bf16 tiles in shared memory, rounded where those round them: the outputs agree bit
+// for bit.
 //
 //   warps 0..7   epilogues, two per TMEM lane quarter: a thread owns 64 of a row's 128
 //                columns; layer-norm statistics of the halves meet in shared memory.
-//                Attention on mma.sync: a 16-row block of whole tokens and one head per warp
-//                and step, probabilities as hi + lo bf16.
+//                Attention on packed fp32: a thread takes one head of two rows of a token.
 //   warp 8       TMA producer: each slot's fp32 vectors, and the weights as 128 x 64 blocks
 //                in the order of the products, through a ring that runs ahead over slots
 //                and tiles.
-//   warp 9       MMA issuer (M = 128, N = 128).
+//   warp 9       MMA issuer (M = 128, N = 128); warps 10 and 11 complete the warpgroup.
 // Epilogues and products alternate through two mbarriers each way (go: operand tiles written,
 // done: accumulators complete); the FFN keeps one 128-column chunk of products ahead.
 // All waits are bounded; the epilogue warps agree on each, so they leave together.
 //
-// What bounds it: the epilogues and the waits between them; a tile's slot takes about 40,000
-// cycles, of which 13,000 in the FFN's GELUs (5,100 are the tanh unit's), 5,200 in the
-// attention, 8,000 in the other epilogues' arithmetic and 9,000 waiting for products (the
-// tensor cores work 7,000). The stages one by one move about 2.2 KB per row and slot through
-// memory in 8 launches a slot; here a slot reads its 128-byte source rows and writes its
-// 256-byte state rows. 8 x 1024 tokens of 12 heads, Top-1 of 2, 4 slots: 2,778 us for the
-// translation staged, 1,098 us with this kernel (987 with the gate, route and projection as they
-// are now); 7,923 ragged tokens of 2 heads, 8 slots:
-// 1,362 and 495 us (375). Steps on the first of these: 16 warps of 32 columns with the vectors read
-// from global memory 1,520 (what L1 the shared memory leaves holds neither them nor spilled
-// registers), vectors staged by the producer and packed fp32 pairs 1,344, attention without
-// integer divisions 1,206, 8 warps of 64 columns 1,214, q ahead of z, v committed apart, the
-// state rows stored behind the next slot's first product and an approximate reciprocal 1,098.
+// What bounds it: the epilogues and the waits between them; a tile's slot takes about 44,000
+// cycles with 12 heads, of which 8,400 in the FFN's GELUs, 10,500 in the attention (6,000 with 2
+// heads), 13,000 in the other epilogues' arithmetic and 12,000 waiting for products or for the
+// slowest warp (the tensor cores work 7,000). The stages one by one move about 2.2 KB per row and
+// slot through memory in 8 launches a slot; here a slot reads its 128-byte source rows and writes
+// its 256-byte state rows. Measured, the translation as a whole: 8 x 1024 tokens of 12 heads, Top-1
+// of 2, 4 slots: 2,778 us by staged kernels, 1,075 us; 7,923 ragged tokens of 2 heads, 8 slots:
+// 1,362 and 376 us. Steps on the first: attention by one thread per row half, its loops over the
+// keys unrolled, 168 registers and 0.5 to 1 KB of spills a thread 1,660; scores in tensor memory and
+// the keys in loops 1,389; registers moved to the epilogue warpgroups (no spills) 1,279; two rows a
+// thread 1,214; loops kept rolled and one call site for each role's wait and copy (the code of a
+// slot, 183 KB, shrinks to 131 KB) 1,064; one row a thread for heads of 64 (their spills) 1,075.
+// Attention on mma.sync with split bf16 weights and products summed in the state's own
+// accumulators took 987 us, but moved outputs by 2e-3 of their norm through other roundings.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "bt_common.cuh"
 #include "gelu.cuh"
@@ -47,23 +48,26 @@ namespace {
 
 constexpr int kScD = 128;                     // row width d
 constexpr int kScEpi = 8;                     // epilogue warps
-constexpr int kScThreads = 32 * (kScEpi + 2);
+constexpr int kScThreads = 32 * (kScEpi + 4);  // three warpgroups: two epilogues, one of roles
+// Registers a thread, per warpgroup: the launch's 168 (65,536 / 384, in eights) moved from the role
+// warps to the epilogues, whose rows of 64 fp32 values and attention would spill.
+constexpr int kScLaunchRegs = 168, kScEpiRegs = 216, kScRoleRegs = 72;
+static_assert(2 * kScEpiRegs + kScRoleRegs <= 3 * kScLaunchRegs, "registers of the launch");
 constexpr int kScBlk = 128 * 128;             // 128 rows x 64 bf16: a weight block, half a row tile
 constexpr int kScTile = 2 * kScBlk;           // 128 rows x 128 bf16
 constexpr int kScXch = 2 * 2 * 128 * 8;       // [parity][column half][row] (mean, M2)
 constexpr int kScMaxRing = 7, kScMinRing = 4; // weight blocks in flight, as many as fit
-// Shared memory: three row tiles, the exchange, bad-token flags, barriers, two slots' vectors,
+// Shared memory: three row tiles, the exchange, barriers, two slots' vectors,
 // the ring.
 constexpr int kScOffXch = 3 * kScTile;
-constexpr int kScOffBad = kScOffXch + kScXch;            // [128] tokens with a non-finite value row
-constexpr int kScOffBars = kScOffBad + 128 * 4;
+constexpr int kScOffBars = kScOffXch + kScXch;
 constexpr int kScOffPrm = kScOffBars + 512;
 constexpr int kScMaxSmem = 232448;
 
 // One slot's fp32 vectors, contiguous (bt_scan_prm_floats): places of each.
 enum PrmAt : int {
   kPrmSIn = 0, kPrmCIn = 128, kPrmLnC = 256, kPrmLnQ = 512, kPrmCQ = 768, kPrmCKv = 896,
-  kPrmHbO = 1152, kPrmLnF = 1280, kPrmHbF = 1536, kPrmLnQn = 1664, kPrmCF1 = 1920
+  kPrmCO = 1152, kPrmLnF = 1280, kPrmCF2 = 1536, kPrmLnQn = 1664, kPrmCF1 = 1920
 };
 __host__ __device__ constexpr int prm_floats(int df) { return kPrmCF1 + df; }
 constexpr int ring_off(int df) { return (kScOffPrm + 2 * prm_floats(df) * 4 + 1023) / 1024 * 1024; }
@@ -111,6 +115,16 @@ __device__ __forceinline__ void ld_pairs(uint32_t addr, uint64_t& a, uint64_t& b
   asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
 }
 
+// Registers of the executing warpgroup's threads, lowered or raised (every warp of it calls).
+template <int N>
+__device__ __forceinline__ void reg_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void reg_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+
 // Barrier id over n threads (n a multiple of 32).
 __device__ __forceinline__ void bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
@@ -154,13 +168,231 @@ __device__ __forceinline__ void add_vec(uint64_t (&v)[32], uint32_t b) {
   }
 }
 
-// Score bits 4 hf + e whose key 8 (e / 2) + 2 tq + e % 2 is below nrow.
-__device__ __forceinline__ uint32_t key_mask(int nrow, int tq) {
-  uint32_t m = 0;
+// The state rows' half in tensor memory: read onto v, and written back.
+__device__ __forceinline__ void add_state(uint32_t addr, uint64_t (&v)[32]) {
 #pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (8 * (e >> 1) + 2 * tq + (e & 1) < nrow) m |= 17u << e;
-  return m;
+  for (int hf = 0; hf < 2; ++hf) {
+    uint32_t u[32];
+    tmem_ld_32x32b_x32(addr + 32 * hf, u);
+    tmem_ld_wait(u);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      v[16 * hf + k] = add2(v[16 * hf + k],
+                            pk(__uint_as_float(u[2 * k]), __uint_as_float(u[2 * k + 1])));
+  }
+}
+__device__ __forceinline__ void store_state(uint32_t addr, const uint64_t (&v)[32]) {
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    uint32_t u[32];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float2 f = unpk(v[16 * hf + k]);
+      u[2 * k] = __float_as_uint(f.x);
+      u[2 * k + 1] = __float_as_uint(f.y);
+    }
+    tmem_st_32x32b_x32(addr + 32 * hf, u);
+  }
+  tmem_st_wait();
+}
+
+__device__ __forceinline__ void unpack8(const uint4& x, float (&f)[8]) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    f[2 * k] = bf16_lo(w[k]);
+    f[2 * k + 1] = bf16_hi(w[k]);
+  }
+}
+
+// Eight 32-bit columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_st8(uint32_t addr, const float (&f)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr),
+               "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]), "f"(f[4]), "f"(f[5]), "f"(f[6]), "f"(f[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t addr, float (&f)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]), "=f"(f[4]), "=f"(f[5]), "=f"(f[6]), "=f"(f[7])
+      : "r"(addr)
+      : "memory");
+}
+
+// Attention of the tile's first n_tok tokens over their own P rows, in fp32 and in the order of
+// bt_attn_kernel: each dot product over its columns in turn, expf of the scaled scores less their
+// maximum, normalised weights, the values added key by key. A thread takes one head of two rows of
+// a token (heads of 64: of one row), so that a key or value is unpacked once for both; four keys to
+// a step, whose scores wait in tensor memory (32 columns at `scratch`, this thread's own), so that
+// the steps are loops. The output replaces the query rows (bf16) in qt; kt and vt: keys and values.
+template <int DH>
+struct Attn {
+  static constexpr int NA = kScD / DH, CH = DH / 8;   // heads; 16-byte pieces of one
+  static constexpr int NR = DH <= 32 ? 2 : 1;         // rows of a thread
+};
+struct AttnTask {   // rows p and p + ceil(P / NR) of a token (its first row rb), the head's first piece
+  int rb, r[2], blk, c0;
+  bool two;         // the second row is one of its own
+};
+template <int DH>
+__device__ __forceinline__ AttnTask attn_task(int task, int P, int tau) {
+  using A = Attn<DH>;
+  const int per = (P + A::NR - 1) / A::NR;
+  const int th = task / per, p0 = task - th * per;
+  const int tok = min(th / A::NA, tau - 1), hd = th % A::NA;
+  const int rb = tok * P, p1 = min(p0 + per, P - 1);
+  return {rb, {rb + p0, rb + p1}, ((hd * A::CH) >> 3) * kScBlk, (hd * A::CH) & 7, p0 + per < P};
+}
+template <int DH>
+__device__ __forceinline__ void attend(uint8_t* qt, const uint8_t* kt, const uint8_t* vt, uint32_t scratch,
+                                       const AttnTask& first, int n_tok, int P, int tau) {
+  constexpr int NA = Attn<DH>::NA, CH = Attn<DH>::CH, NR = Attn<DH>::NR;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float scale = rsqrtf(static_cast<float>(DH));
+  const int n_task = n_tok * NA * ((P + NR - 1) / NR);
+#pragma unroll 1
+  for (int t0 = warp * 32; t0 < n_task; t0 += 32 * kScEpi) {
+    const AttnTask t = t0 == warp * 32 ? first : attn_task<DH>(t0 + lane, P, tau);
+    auto at = [&](int r, int c) { return t.blk + r * 128 + (((t.c0 + c) ^ (r & 7)) << 4); };
+    auto piece = [&](const uint8_t* tile, int r, int c) {
+      return *reinterpret_cast<const uint4*>(tile + at(r, c));
+    };
+    __syncwarp();
+    float m[NR];
+#pragma unroll
+    for (int n = 0; n < NR; ++n) m[n] = -INFINITY;
+    {
+      uint64_t q[NR][DH];   // each value twice: two keys take the halves of packed fp32
+#pragma unroll
+      for (int n = 0; n < NR; ++n)
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+          float f[8];
+          unpack8(piece(qt, t.r[n], c), f);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) q[n][8 * c + k] = pk(f[k], f[k]);
+        }
+#pragma unroll 1
+      for (int j0 = 0; j0 < P; j0 += 4) {
+        uint64_t s[NR][2];   // keys j0 + 2 h and j0 + 2 h + 1
+#pragma unroll
+        for (int n = 0; n < NR; ++n) s[n][0] = s[n][1] = 0ull;
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+          float f[4][8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) unpack8(piece(kt, t.rb + min(j0 + i, P - 1), c), f[i]);
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const uint64_t kk = pk(f[2 * h][k], f[2 * h + 1][k]);
+#pragma unroll
+              for (int n = 0; n < NR; ++n) s[n][h] = fma2(q[n][8 * c + k], kk, s[n][h]);
+            }
+        }
+        float x[8];   // x[2 i + n]: key j0 + i, row n
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float2 y = unpk(s[n % NR][h]);
+            x[4 * h + n] = y.x * scale;
+            x[4 * h + 2 + n] = y.y * scale;
+          }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (j0 + i < P)
+#pragma unroll
+            for (int n = 0; n < NR; ++n) m[n] = fmaxf(m[n], x[2 * i + n]);
+        tmem_st8(scratch + 2 * j0, x);
+      }
+    }
+    tmem_st_wait();
+    float inv[NR];
+#pragma unroll
+    for (int n = 0; n < NR; ++n) inv[n] = 0.f;   // the sums first
+#pragma unroll 1
+    for (int j0 = 0; j0 < P; j0 += 4) {
+      float x[8];
+      tmem_ld8(scratch + 2 * j0, x);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int n = 0; n < NR; ++n) {
+          x[2 * i + n] = expf(x[2 * i + n] - m[n]);
+          if (j0 + i < P) inv[n] += x[2 * i + n];
+        }
+      tmem_st8(scratch + 2 * j0, x);
+    }
+    tmem_st_wait();
+    uint64_t o[NR][DH / 2];
+#pragma unroll
+    for (int n = 0; n < NR; ++n) {
+      inv[n] = 1.f / inv[n];
+#pragma unroll
+      for (int k = 0; k < DH / 2; ++k) o[n][k] = 0ull;
+    }
+#pragma unroll 1
+    for (int j0 = 0; j0 < P; j0 += 4) {
+      float x[8];
+      tmem_ld8(scratch + 2 * j0, x);
+      auto step = [&](auto whole) {   // four keys, or the last P - j0
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+          uint4 u[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            u[i] = piece(vt, t.rb + (decltype(whole)::value ? j0 + i : min(j0 + i, P - 1)), c);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (!decltype(whole)::value && j0 + i >= P) break;
+            float f[8];
+            unpack8(u[i], f);
+#pragma unroll
+            for (int n = 0; n < NR; ++n) {
+              const float w = x[2 * i + n] * inv[n];
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                o[n][4 * c + k] = fma2(pk(w, w), pk(f[2 * k], f[2 * k + 1]), o[n][4 * c + k]);
+            }
+          }
+        }
+      };
+      if (j0 + 4 <= P) step(std::true_type{});
+      else step(std::false_type{});
+    }
+    if (t0 + lane < n_task) {
+#pragma unroll
+      for (int n = 0; n < NR; ++n) {
+        if (n == 1 && !t.two) break;
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+          uint32_t u[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float2 f = unpk(o[n][4 * c + k]);
+            u[k] = pack2(f.x, f.y);
+          }
+          *reinterpret_cast<uint4*>(qt + at(t.r[n], c)) = make_uint4(u[0], u[1], u[2], u[3]);
+        }
+      }
+    }
+  }
+}
+
+// The products of a slot, in order; from kStF on those of the FFN.
+enum Stage : int { kStIn = 0, kStQ, kStK, kStV, kStO, kStF };
+struct FfnStage {
+  bool first;   // W_F1 of hidden chunk hc, else W_F2 of it
+  int hc;
+};
+// W_F1 of chunks 0 and 1, then W_F2 of a chunk and W_F1 two chunks on, in turn (2 n_hc products).
+__device__ __forceinline__ FfnStage ffn_stage(int i, int n_hc) {
+  if (i == 2 * n_hc - 1) return {false, n_hc - 1};
+  if (i == 0 || (i & 1)) return {true, (i + 1) >> 1};
+  return {false, (i >> 1) - 1};
 }
 
 // NXV: 16-byte pieces of a source row per thread (d_s / 16); DH: attention head width.
@@ -179,7 +411,6 @@ __global__ void __launch_bounds__(kScThreads, 1)
   uint8_t* sRing = smem + ring_at;
   const uint32_t sPrm = smem_u32(smem + kScOffPrm);
   float2* xch = reinterpret_cast<float2*>(smem + kScOffXch);
-  int* bad = reinterpret_cast<int*>(smem + kScOffBad);
   uint64_t* wfull = reinterpret_cast<uint64_t*>(smem + kScOffBars);   // [ring]
   uint64_t* wempty = wfull + kScMaxRing;
   uint64_t* pfull = wempty + kScMaxRing;   // [2] a slot's vectors landed
@@ -223,138 +454,143 @@ __global__ void __launch_bounds__(kScThreads, 1)
   uint32_t issued_mask = 0, issue_parity = 0, prm_issued = 0, prm_parity = 0;
   bool mma_issued = false;
 
-  if (warp == kScEpi) {
-    if (lane == 0) {
-      // ------------------------------------------------ weights
+  if (warp >= kScEpi) {
+    reg_dec<kScRoleRegs>();   // the role warpgroup, its two idle warps included
+    if (warp == kScEpi) {
+      if (lane == 0) {
+        // ------------------------------------------------ weights
+        int slot = 0;
+        uint32_t phase = 0, n_prm = 0;
+        bool ok = true;
+        auto put = [&](const CUtensorMap* map, int k0, int row) {
+          if (!ok) return;
+          if (!mbar_wait(&wempty[slot], phase ^ 1u, abort_flag, wl)) {
+            ok = false;
+            return;
+          }
+          mbar_arrive_expect_tx(&wfull[slot], kScBlk);
+          tma_load_2d(sRing + slot * kScBlk, map, &wfull[slot], k0, row);
+          issued_mask |= 1u << slot;
+          issue_parity = (issue_parity & ~(1u << slot)) | (phase << slot);
+          if (++slot == n_ring) {
+            slot = 0;
+            phase ^= 1u;
+          }
+        };
+        for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
+          const Work w = decode(a, c, it);
+          if (!w.active) continue;
+#pragma unroll 1
+          for (int r = 0; r < d.N && ok; ++r) {
+            const int gr = w.g * d.N + r;
+            if (!mbar_wait(&pempty[n_prm & 1], ((n_prm >> 1) & 1) ^ 1u, abort_flag, wl)) {
+              ok = false;
+              break;
+            }
+            mbar_arrive_expect_tx(&pfull[n_prm & 1], prm_bytes);
+            bulk_load(sPrm + (n_prm & 1) * prm_bytes, a.prm + int64_t(gr) * prm_floats(d.df), prm_bytes,
+                      &pfull[n_prm & 1]);
+            prm_issued |= 1u << (n_prm & 1);
+            prm_parity = (prm_parity & ~(1u << (n_prm & 1))) | (((n_prm >> 1) & 1) << (n_prm & 1));
+            ++n_prm;
+#pragma unroll 1
+            for (int st = 0; st < kStF + 2 * n_hc; ++st) {
+              const CUtensorMap* map = st == kStIn ? &tmWin : st == kStQ ? &tmWq : st == kStO ? &tmWo : &tmWkv;
+              int k0 = 0, row = st == kStIn ? w.g * D : st == kStK || st == kStV ? (2 * gr + st - kStK) * D : gr * D;
+              if (st >= kStF) {
+                const FfnStage f = ffn_stage(st - kStF, n_hc);
+                map = f.first ? &tmWf1 : &tmWf2;
+                if (f.first) row = gr * d.df + f.hc * 128;
+                else k0 = f.hc * 128;
+              }
+#pragma unroll 1
+              for (int kb = 0; kb < (st == kStIn ? 2 * DS / 64 : 2); ++kb) put(map, k0 + 64 * kb, row);
+            }
+          }
+        }
+      }
+    } else if (warp == kScEpi + 1) {
+      // ------------------------------------------------ MMA issuer (warp-uniform, elected lane)
+      const uint32_t idesc = idesc_bf16_f32(128, 128);
       int slot = 0;
-      uint32_t phase = 0, n_prm = 0;
+      uint32_t phase = 0, n_go = 0, n_done = 0;
       bool ok = true;
-      auto put = [&](const CUtensorMap& map, int k0, int row) {
-        if (!ok) return;
-        if (!mbar_wait(&wempty[slot], phase ^ 1u, abort_flag, wl)) {
-          ok = false;
-          return;
-        }
-        mbar_arrive_expect_tx(&wfull[slot], kScBlk);
-        tma_load_2d(sRing + slot * kScBlk, &map, &wfull[slot], k0, row);
-        issued_mask |= 1u << slot;
-        issue_parity = (issue_parity & ~(1u << slot)) | (phase << slot);
-        if (++slot == n_ring) {
-          slot = 0;
-          phase ^= 1u;
-        }
-      };
       for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
         const Work w = decode(a, c, it);
         if (!w.active) continue;
+#pragma unroll 1
         for (int r = 0; r < d.N && ok; ++r) {
-          const int gr = w.g * d.N + r;
-          if (!mbar_wait(&pempty[n_prm & 1], ((n_prm >> 1) & 1) ^ 1u, abort_flag, wl)) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&pfull[n_prm & 1], prm_bytes);
-          bulk_load(sPrm + (n_prm & 1) * prm_bytes, a.prm + int64_t(gr) * prm_floats(d.df), prm_bytes,
-                    &pfull[n_prm & 1]);
-          prm_issued |= 1u << (n_prm & 1);
-          prm_parity = (prm_parity & ~(1u << (n_prm & 1))) | (((n_prm >> 1) & 1) << (n_prm & 1));
-          ++n_prm;
-          for (int kb = 0; kb < 2 * DS / 64; ++kb) put(tmWin, 64 * kb, w.g * D);
-          for (int kb = 0; kb < 2; ++kb) put(tmWq, 64 * kb, gr * D);
-          for (int n = 0; n < 2; ++n)
-            for (int kb = 0; kb < 2; ++kb) put(tmWkv, 64 * kb, gr * 2 * D + n * D);
-          for (int kb = 0; kb < 2; ++kb) put(tmWo, 64 * kb, gr * D);
-          auto f1 = [&](int hc) {
-            for (int kb = 0; kb < 2; ++kb) put(tmWf1, 64 * kb, gr * d.df + hc * 128);
-          };
-          f1(0);
-          if (n_hc > 1) f1(1);
-          for (int hc = 0; hc < n_hc; ++hc) {
-            for (int kb = 0; kb < 2; ++kb) put(tmWf2, hc * 128 + 64 * kb, gr * D);
-            if (hc + 2 < n_hc) f1(hc + 2);
-          }
-        }
-      }
-    }
-  } else if (warp == kScEpi + 1) {
-    // ------------------------------------------------ MMA issuer (warp-uniform, elected lane)
-    const uint32_t idesc = idesc_bf16_f32(128, 128);
-    int slot = 0;
-    uint32_t phase = 0, n_go = 0, n_done = 0;
-    bool ok = true;
-    auto wait_go = [&]() {
-      if (ok && !mbar_wait(&go[n_go & 1], (n_go >> 1) & 1, abort_flag, wl)) ok = false;
-      ++n_go;
-      tc_fence_after();
-    };
-    // `units` weight blocks against the A tile's 64-column blocks (unit u: block u % nblk)
-    auto product = [&](uint32_t acc, uint32_t a_tile, int nblk, int units, bool onto) {
-      for (int u = 0; u < units && ok; ++u) {
-        if (!mbar_wait(&wfull[slot], phase, abort_flag, wl)) {
-          ok = false;
-          return;
-        }
-        tc_fence_after();
-        const uint64_t ad = sdesc_k_sw128(a_tile + (u % nblk) * kScBlk);
-        const uint64_t bd = sdesc_k_sw128(smem_u32(sRing + slot * kScBlk));
-        if (elect_one()) {
+#pragma unroll 1
+          for (int st = 0; st < kStF + 2 * n_hc && ok; ++st) {
+            uint32_t acc = 128, tile = sXQ;
+            bool go_first = false, commit = true, onto = false;
+            switch (st) {
+              case kStIn: tile = sKB; go_first = true; break;   // hi, then lo, x source rows
+              case kStQ: acc = 256; go_first = r == 0; commit = false; break;   // r > 0: rows of the slot before
+              case kStK: acc = 384; tile = sXZ; go_first = r > 0; break;
+              case kStV: tile = sXZ; break;
+              case kStO: go_first = true; break;
+              default: {
+                const FfnStage f = ffn_stage(st - kStF, n_hc);
+                if (f.first) {
+                  acc = 128 + 128 * (f.hc & 1);
+                  go_first = f.hc == 0;
+                } else {
+                  acc = 384;
+                  tile = (f.hc & 1) ? sKB : sXZ;
+                  go_first = true;
+                  commit = f.hc == n_hc - 1;
+                  onto = f.hc > 0;
+                }
+              }
+            }
+            if (go_first) {
+              if (!mbar_wait(&go[n_go & 1], (n_go >> 1) & 1, abort_flag, wl)) ok = false;
+              ++n_go;
+              tc_fence_after();
+            }
+            const int nblk = st == kStIn ? DS / 64 : 2, units = st == kStIn ? 2 * DS / 64 : 2;
+            // `units` weight blocks against the A tile's 64-column blocks (1 or 2 of them, in turn)
+#pragma unroll 1
+            for (int u = 0; u < units && ok; ++u) {
+              if (!mbar_wait(&wfull[slot], phase, abort_flag, wl)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint64_t ad = sdesc_k_sw128(tile + (u & (nblk - 1)) * kScBlk);
+              const uint64_t bd = sdesc_k_sw128(smem_u32(sRing + slot * kScBlk));
+              if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma_bf16(tmem + acc, ad + 2 * k, bd + 2 * k, idesc, onto || (u | k) != 0);
-          umma_commit(&wempty[slot]);
+                for (int k = 0; k < 4; ++k)
+                  umma_bf16(tmem + acc, ad + 2 * k, bd + 2 * k, idesc, onto || (u | k) != 0);
+                umma_commit(&wempty[slot]);
+              }
+              __syncwarp();
+              mma_issued = true;
+              if (++slot == n_ring) {
+                slot = 0;
+                phase ^= 1u;
+              }
+            }
+            if (commit) {
+              if (ok && elect_one()) umma_commit(&done[n_done & 1]);
+              __syncwarp();
+              ++n_done;
+            }
+          }
         }
-        __syncwarp();
-        mma_issued = true;
-        if (++slot == n_ring) {
-          slot = 0;
-          phase ^= 1u;
-        }
-      }
-    };
-    auto finish = [&]() {
-      if (ok && elect_one()) umma_commit(&done[n_done & 1]);
-      __syncwarp();
-      ++n_done;
-    };
-    for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
-      const Work w = decode(a, c, it);
-      if (!w.active) continue;
-      for (int r = 0; r < d.N && ok; ++r) {
-        wait_go();
-        product(128, sKB, DS / 64, 2 * DS / 64, false);   // W_in hi, then lo, x source rows
-        finish();
-        if (r > 0) product(256, sXQ, 2, 2, false);   // q needs the earlier slot's rows only
-        wait_go();
-        if (r == 0) product(256, sXQ, 2, 2, false);
-        product(384, sXZ, 2, 2, false);
-        finish();
-        product(128, sXZ, 2, 2, false);
-        finish();
-        wait_go();
-        product(0, sXQ, 2, 2, true);   // h += W_O o
-        finish();
-        wait_go();
-        auto f1 = [&](int hc) {
-          product(128 + 128 * (hc & 1), sXQ, 2, 2, false);
-          finish();
-        };
-        f1(0);
-        if (n_hc > 1) f1(1);
-        for (int hc = 0; hc < n_hc && ok; ++hc) {
-          wait_go();
-          product(0, (hc & 1) ? sKB : sXZ, 2, 2, true);   // h += W_F2 f
-          if (hc + 2 < n_hc) f1(hc + 2);
-        }
-        finish();
       }
     }
   } else {
+    reg_inc<kScEpiRegs>();
     // ------------------------------------------------ epilogues
     const int q = warp & 3, cg = warp >> 2;
     const int row = q * 32 + lane;
     const int col0 = 64 * cg;
     const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
     const int t = row / d.P, p = row - t * d.P;
+    const AttnTask task = attn_task<DH>(threadIdx.x, d.P, d.tau);
     uint32_t n_go = 0, n_done = 0, n_prm = 0, xpar = 0;
     bool ok = true;
     auto ready = [&]() {   // this warp's operand rows are written, its accumulator reads are done
@@ -384,25 +620,24 @@ __global__ void __launch_bounds__(kScThreads, 1)
       m2 = (m2 + o.y) + e * e * (0.5f * n);
       mean = 0.5f * (mean + o.x);
     };
+    // sums in column order, as row_stats of bt.cu
     auto stats = [&](const uint64_t (&v)[32], float& mean, float& m2) {
-      uint64_t s0 = v[0], s1 = v[1];
+      float sum = 0.f;
 #pragma unroll
-      for (int k = 2; k < 32; k += 2) {
-        s0 = add2(s0, v[k]);
-        s1 = add2(s1, v[k + 1]);
+      for (int k = 0; k < 32; ++k) {
+        const float2 f = unpk(v[k]);
+        sum += f.x;
+        sum += f.y;
       }
-      const float2 f = unpk(add2(s0, s1));
-      mean = (f.x + f.y) * (1.f / 64);
+      mean = sum * (1.f / 64);
       const uint64_t nm = pk(-mean, -mean);
-      s0 = s1 = 0ull;
+      m2 = 0.f;
 #pragma unroll
-      for (int k = 0; k < 32; k += 2) {
-        const uint64_t e0 = add2(v[k], nm), e1 = add2(v[k + 1], nm);
-        s0 = fma2(e0, e0, s0);
-        s1 = fma2(e1, e1, s1);
+      for (int k = 0; k < 32; ++k) {
+        const float2 f = unpk(add2(v[k], nm));
+        m2 = fmaf(f.x, f.x, m2);
+        m2 = fmaf(f.y, f.y, m2);
       }
-      const float2 q2 = unpk(add2(s0, s1));
-      m2 = q2.x + q2.y;
       combine(64.f, mean, m2);
     };
     // tile <- bf16(gamma (v - mean) rstd + beta)
@@ -482,37 +717,43 @@ __global__ void __launch_bounds__(kScThreads, 1)
     const uint4* src = nullptr;
     if (it < total) load_x(src = source(w), 0);
     while (it < total && ok) {
-      const int vrows = valid_rows(w);
+      const int vrows = valid_rows(w), n_tok = vrows / d.P;
       const int64_t row0 = int64_t(w.g) * d.R + w.row0;   // the tile's first row (token-major)
       int it_n = it;
+#pragma unroll 1
       for (int r = 0; r < d.N && ok; ++r) {
         // ---- source rows into the A tile, and their statistics
-        float mu, m2x;
-        {
-          float s = 0.f;
 #pragma unroll
-          for (int i = 0; i < NXV; ++i)
-            s += ((bf16_lo(xv[i].x) + bf16_hi(xv[i].x)) + (bf16_lo(xv[i].y) + bf16_hi(xv[i].y))) +
-                 ((bf16_lo(xv[i].z) + bf16_hi(xv[i].z)) + (bf16_lo(xv[i].w) + bf16_hi(xv[i].w)));
-          mu = s * (2.f / DS);
-          m2x = 0.f;
-#pragma unroll
-          for (int i = 0; i < NXV; ++i) {
-            const uint32_t u[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float lo = bf16_lo(u[e]) - mu, hi = bf16_hi(u[e]) - mu;
-              m2x = fmaf(lo, lo, fmaf(hi, hi, m2x));
-            }
-            const int ch = cg * NXV + i;   // 16-byte piece of the row
-            st_shared_v4(sKB + (ch >> 3) * kScBlk + row * 128 + (((ch & 7) ^ (row & 7)) << 4), u[0],
-                         u[1], u[2], u[3]);
-          }
+        for (int i = 0; i < NXV; ++i) {
+          const int ch = cg * NXV + i;   // 16-byte piece of the row
+          st_shared_v4(sKB + (ch >> 3) * kScBlk + row * 128 + (((ch & 7) ^ (row & 7)) << 4), xv[i].x,
+                       xv[i].y, xv[i].z, xv[i].w);
         }
-        if (cg == 0) bad[row] = 0;
         ready();
         rows_out();   // while the product runs; the next write to sXZ comes after its wait
-        combine(DS / 2, mu, m2x);
+        bar_sync(2 + q, 64);   // both halves of the row are in the tile
+        auto piece = [&](int ch) {
+          return ld_shared_v4(sKB + (ch >> 3) * kScBlk + row * 128 + (((ch & 7) ^ (row & 7)) << 4));
+        };
+        float mu = 0.f, m2x = 0.f;
+#pragma unroll
+        for (int ch = 0; ch < 2 * NXV; ++ch) {
+          const uint4 u = piece(ch);
+          mu += bf16_lo(u.x) + bf16_hi(u.x) + bf16_lo(u.y) + bf16_hi(u.y) + bf16_lo(u.z) +
+                bf16_hi(u.z) + bf16_lo(u.w) + bf16_hi(u.w);
+        }
+        mu *= 1.f / DS;
+#pragma unroll
+        for (int ch = 0; ch < 2 * NXV; ++ch) {
+          const uint4 u = piece(ch);
+          const uint32_t uw[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float lo = bf16_lo(uw[e]) - mu, hi = bf16_hi(uw[e]) - mu;
+            m2x = fmaf(lo, lo, m2x);
+            m2x = fmaf(hi, hi, m2x);
+          }
+        }
         const float rsx = rsqrtf(m2x * (1.f / DS) + kLnEps);
         // ---- z = GELU(LN-folded W_in x + c); LN_C(z); slot 0: h = z, LN_Q(h)
         if (lane == 0) mbar_wait(&pfull[n_prm & 1], (n_prm >> 1) & 1, abort_flag, wl);
@@ -539,18 +780,7 @@ __global__ void __launch_bounds__(kScThreads, 1)
           const float rstd = rsqrtf(m2 * (1.f / D) + kLnEps);
           store_ln(sXZ, v, mean, rstd, prm + kPrmLnC * 4);
           if (r == 0) {
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              uint32_t u[32];
-#pragma unroll
-              for (int k = 0; k < 16; ++k) {
-                const float2 f = unpk(v[16 * hf + k]);
-                u[2 * k] = __float_as_uint(f.x);
-                u[2 * k + 1] = __float_as_uint(f.y);
-              }
-              tmem_st_32x32b_x32(tmem + lanes + col0 + 32 * hf, u);
-            }
-            tmem_st_wait();
+            store_state(tmem + lanes + col0, v);
             store_ln(sXQ, v, mean, rstd, prm + kPrmLnQ * 4);
           }
         }
@@ -566,114 +796,18 @@ __global__ void __launch_bounds__(kScThreads, 1)
         if (!wait_done()) break;
         load_acc(tmem + lanes + 128 + col0, v);
         add_vec(v, prm + (kPrmCKv + D + col0) * 4);
-        {
-          // a non-finite value row spoils its own token only: it enters the shared products of a
-          // 16-row block as zeros, and the token's outputs become NaN
-          uint64_t nf = 0ull;
-#pragma unroll
-          for (int k = 0; k < 32; ++k) nf = fma2(v[k], 0ull, nf);
-          const float2 f = unpk(nf);
-          if (f.x + f.y != 0.f) {   // NaN
-            bad[t] = 1;
-#pragma unroll
-            for (int k = 0; k < 32; ++k) v[k] = 0ull;
-          }
-        }
         store_row64(sXZ, row, cg, v);
         bar_sync(1, 32 * kScEpi);
-        // ---- attention: blocks of floor(16 / P) whole tokens x heads over the warps
-        {
-          constexpr int KS = DH / 16, CH = DH / 8, NA = D / DH;   // K steps; 16-byte chunks; heads
-          // attention blocks of tb whole tokens (at most 16 rows); this lane's score rows gq, gq + 8
-          // and keys 8 (e / 2) + 2 tq + e % 2 within a block, and which pairs share a token
-          const int P = d.P, ln = lane;
-          const int tb = 16 / P, tbP = tb * P, tauP = d.tau * P, nblk = (d.tau + tb - 1) / tb;
-          const int mi = ln >> 3, ri = ln & 7, gq = ln >> 2, tq = ln & 3;
-          const int it0 = gq / P, it1 = (gq + 8) / P;
-          uint32_t same = 0;
-      #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int kt = (8 * (e >> 1) + 2 * tq + (e & 1)) / P;
-            same |= (kt == it0 ? 1u : 0u) << e | (kt == it1 ? 16u : 0u) << e;
-          }
-          const float sl2 = rsqrtf(float(DH)) * 1.4426950408889634f;
-          for (int task = warp; task < nblk * NA; task += kScEpi) {
-            __syncwarp();
-            const int blk = task / NA, hd = task % NA;
-            const int rb = blk * tbP, nrow = min(tbP, tauP - rb);
-            // chunk k of this head in row rb + i (k = 0 here: an XOR of its bits reaches the others)
-            const uint32_t hoff = ((hd * CH) >> 3) * kScBlk, hc0 = (hd * CH) & 7;
-            auto at = [&](uint32_t tile, int i) -> uint32_t {
-              const uint32_t rr = rb + min(i, nrow - 1);
-              return tile + hoff + rr * 128 + ((hc0 ^ (rr & 7)) << 4);
-            };
-            const uint32_t qa = at(sXQ, ri + 8 * (mi & 1)), ka = at(sKB, ri + 8 * (mi >> 1));
-            const uint32_t va = qa + (sXZ - sXQ);
-            float s[2][4];
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) s[j][e] = 0.f;
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-              uint32_t aq[4], bk[4];
-              ldsm4(qa ^ ((2 * ks + (mi >> 1)) << 4), aq);
-              ldsm4(ka ^ ((2 * ks + (mi & 1)) << 4), bk);
-              mma_bf16(s[0], aq[0], aq[1], aq[2], aq[3], bk[0], bk[1]);
-              mma_bf16(s[1], aq[0], aq[1], aq[2], aq[3], bk[2], bk[3]);
-            }
-            // pairs of one token, among the block's rows
-            const uint32_t ok8 = same & (nrow >= 16 ? 0xFFu : key_mask(nrow, tq));
-            uint32_t ph[2][2], pl[2][2];   // [n tile][row half]
-            float inv[2];
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              float x[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e)   // key 8 (e / 2) + 2 tq + e % 2
-                x[e] = (ok8 >> (4 * hf + e) & 1u) ? s[e >> 1][2 * hf + (e & 1)] : -INFINITY;
-              float mx = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
-              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-              mx = gq + 8 * hf < nrow ? mx * sl2 : 0.f;   // rows past the block: every key masked
-#pragma unroll
-              for (int e = 0; e < 4; ++e) x[e] = ex2_fast(fmaf(x[e], sl2, -mx));
-              float den = (x[0] + x[1]) + (x[2] + x[3]);
-              den += __shfl_xor_sync(0xffffffffu, den, 1);
-              den += __shfl_xor_sync(0xffffffffu, den, 2);
-              inv[hf] = __fdividef(1.f, den);   // 1 <= den <= 16 on the rows that are kept
-#pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                const uint32_t hi = pack2(x[2 * j], x[2 * j + 1]);
-                ph[j][hf] = hi;
-                pl[j][hf] = pack2(x[2 * j] - bf16_lo(hi), x[2 * j + 1] - bf16_hi(hi));
-              }
-            }
-            const bool in0 = gq < nrow, in1 = gq + 8 < nrow;
-            if (in0 && bad[blk * tb + it0]) inv[0] = __uint_as_float(0x7FC00000u);
-            if (in1 && bad[blk * tb + it1]) inv[1] = __uint_as_float(0x7FC00000u);
-            const uint32_t o0 = at(sXQ, gq) + 4 * tq, o1 = at(sXQ, gq + 8) + 4 * tq;
-#pragma unroll
-            for (int ch = 0; ch < CH; ch += 2) {
-              uint32_t bv[4];
-              __syncwarp();
-              ldsm4_t(va ^ ((ch + (mi >> 1)) << 4), bv);
-#pragma unroll
-              for (int n = 0; n < 2; ++n) {
-                float o[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_bf16(o, ph[0][0], ph[0][1], ph[1][0], ph[1][1], bv[2 * n], bv[2 * n + 1]);
-                mma_bf16(o, pl[0][0], pl[0][1], pl[1][0], pl[1][1], bv[2 * n], bv[2 * n + 1]);
-                if (in0) st_shared_u32(o0 ^ ((ch + n) << 4), pack2(o[0] * inv[0], o[1] * inv[0]));
-                if (in1) st_shared_u32(o1 ^ ((ch + n) << 4), pack2(o[2] * inv[1], o[3] * inv[1]));
-              }
-            }
-          }
-        }
+        // ---- attention over each token's rows
+        attend<DH>(smem, smem + 2 * kScTile, smem + kScTile, tmem + lanes + 128 + col0, task,
+                   n_tok, d.P, d.tau);
         ready();
         // ---- LN_F(h) of h += W_O o + b_O
         if (!wait_done()) break;
-        load_acc(tmem + lanes + col0, v);
-        add_vec(v, prm + (kPrmHbO + col0) * 4);
+        load_acc(tmem + lanes + 128 + col0, v);
+        add_vec(v, prm + (kPrmCO + col0) * 4);
+        add_state(tmem + lanes + col0, v);
+        store_state(tmem + lanes + col0, v);
         stats(v, mean, m2);
         store_ln(sXQ, v, mean, rsqrtf(m2 * (1.f / D) + kLnEps), prm + kPrmLnF * 4);
         ready();
@@ -685,6 +819,7 @@ __global__ void __launch_bounds__(kScThreads, 1)
           if (it_n < total) load_x(src = source(w), 0);
         }
         // ---- FFN hidden chunks
+#pragma unroll 1
         for (int hc = 0; hc < n_hc; ++hc) {
           if (!wait_done()) break;
           load_acc(tmem + lanes + 128 + 128 * (hc & 1) + col0, v);
@@ -696,8 +831,10 @@ __global__ void __launch_bounds__(kScThreads, 1)
         }
         // ---- h_r: statistics for LN_out, rows out, LN_Q for the next slot
         if (!ok || !wait_done()) break;
-        load_acc(tmem + lanes + col0, v);
-        add_vec(v, prm + (kPrmHbF + col0) * 4);
+        load_acc(tmem + lanes + 384 + col0, v);
+        add_vec(v, prm + (kPrmCF2 + col0) * 4);
+        add_state(tmem + lanes + col0, v);
+        if (r + 1 < d.N) store_state(tmem + lanes + col0, v);
         store_row64(sXZ, row, cg, v);
         stats(v, mean, m2);   // its barrier covers this lane quarter's rows of sXZ too
         const int64_t slot_row = int64_t(r) * d.G * d.R;
@@ -794,16 +931,8 @@ void bt_scan_pack_prm(const BtDims& d, const BtScanVecs& v, int g, int slot, flo
   put(kPrmLnF, v.ln_f + gr * 2 * D, 2 * D);
   put(kPrmLnQn, v.ln_q + (slot + 1 < d.N ? gr + 1 : gr) * 2 * D, 2 * D);
   put(kPrmCF1, v.c_f1 + gr * d.df, d.df);
-  // the biases that the state accumulator leaves out: b_O and b_F2 of the slots so far
-  for (size_t k = 0; k < D; ++k) {
-    double sum = 0.0;
-    for (int r = 0; r <= slot; ++r) {
-      if (r > 0) sum += v.c_f2[(size_t(g) * d.N + r - 1) * D + k];
-      sum += v.c_o[(size_t(g) * d.N + r) * D + k];
-    }
-    out[kPrmHbO + k] = float(sum);
-    out[kPrmHbF + k] = float(sum + v.c_f2[gr * D + k]);
-  }
+  put(kPrmCO, v.c_o + gr * D, D);
+  put(kPrmCF2, v.c_f2 + gr * D, D);
 }
 
 // Rows of 128 (one 128-column tile of state), an FFN in whole 128-column chunks whose vectors

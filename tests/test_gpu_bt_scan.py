@@ -79,6 +79,28 @@ def test_scan_matches_oracle(name):
                 assert bool((G.int_view(dst)[l] == s).all())
 
 
+# more edges: tokens of one row, of two with a longer window, of three and of 13 (one row stays alone)
+SAME = dict(SHAPES, **{
+    "p2_dh32": (2, 64, 2, 32, 2, 1, (65, 64, 1), (0, 8, 128, 4, 256)),
+    "p13_dh64": (13, 128, 2, 32, 2, 0, (9, 10), (1, 3, 128, 2, 128)),
+    "p3_dh16": (3, 64, 4, 32, 3, 1, (43, 42, 85), (0, 4, 128, 8, 512)),
+    "p1_dh64": (1, 64, 2, 64, 1, 0, (128, 200), (0, 3, 128, 2, 2048)),
+})
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+@pytest.mark.parametrize("name", sorted(SAME))
+def test_scan_equals_the_staged_kernels_bit_for_bit(name, seed):
+    """The same fp32 sums in the same order, rounded to bf16 at the same places."""
+    P, ds, ht, dt, e, top_k, lens, bt = SAME[name]
+    wl = W(name, 3, P, ds, bt[0] + bt[1] + 1, ht, dt, e, 0, len(lens), max(lens), "bf16", lens, top_k=top_k, bt=bt)
+    ins = _inputs(wl, seed)
+    scan, staged = _run(wl, *ins), _run(wl, *ins, staged=True)
+    assert scan[2] < staged[2]
+    for a, b in zip(scan[:2], staged[:2]):
+        assert torch.equal(G.int_view(a), G.int_view(b))
+
+
 def test_scan_keeps_non_finite_tokens_apart():
     """A NaN or infinity in one token's rows makes that token's outputs NaN and leaves every
     other token as it was, also those that share its attention blocks."""
