@@ -22,19 +22,25 @@
 // 252 us as three tcgen05 lanes, 248 us with the MMA fragments loaded straight from global
 // memory (each 16-byte load instruction touches 4 to 8 rows: 1,650 L1 wavefronts per item),
 // 177 us with this ring and a general tile cursor (3,200 instructions per item), 162 us
-// with the static tile stream (1,550), 142 us with the item and tile orders below. The
-// shapes that ran on CUDA cores: 8 x 1024 positions, 12 heads of 64, S = 128: 693 to
-// 209 us; 4 x 4096, S = 256, d = 128: 1,127 to 245 us; full causal layers of 2047 + 1025
-// positions: 980 to 200 us.
+// with the static tile stream (1,550), 142 to 151 us with the item and tile orders below (by run).
+//
+// Probabilities that the CUDA-core kernel before this one held in fp32 (heads of 64, sets past
+// 128 rows, full layers) stay fp32: three bf16 parts, exact. Two parts rounded to 2^-17 moved the
+// error against 64 bits from 1.630332e-3 to 1.630333e-3; with three it is the
+// former kernel's to eight digits, with the small parts added apart from the large one where they
+// take MMAs of their own (three sums into one accumulator over 1,500 rows: + 2e-10). Whole calls,
+// CUDA cores, two parts, three: 8 x 1024 positions, 12 heads of 64, S = 128: 739, 227, 227 us;
+// 4 x 4096, 12 heads of 128 on 2, S = 256: 296 and 328 us (1,127 us for the former kernel alone); full causal
+// layers of 2047 + 1025 positions, the same heads: 231 and 279 us (980).
 #include "replay_common.cuh"
 
 namespace mot {
 namespace {
 
-// How a probability enters the second product: as bf16; or as the sum of two bf16 (hi +
-// lo, relative error 2^-17), the halves in different columns (groups of at most 4 heads:
-// no extra MMA) or in two MMAs.
-enum ProbForm : int { kProbBf16 = 0, kProbSplitCols = 1, kProbSplitMma = 2 };
+// How a probability enters the second product: as bf16; or as the sum of three bf16 (hi + mid +
+// lo: its fp32, exactly), the parts of one or two heads in different columns (no extra MMA),
+// of 3 or 4 heads two parts in columns and one in a second MMA, else in three MMAs.
+enum ProbForm : int { kProbBf16 = 0, kProbCols1 = 1, kProbCols2 = 2, kProbCols4 = 4, kProbMma3 = 8 };
 
 constexpr int kRgStages = 4;
 constexpr int kRgTile = 4096;
@@ -69,6 +75,15 @@ __device__ __forceinline__ uint32_t movm_t(uint32_t x) {
 
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
+// fp32 as three bf16 without rounding: the upper half of x holds 8 of its 24 significant bits, that of
+// what is left below it (exact) the next 8 from its leading one, and what is below those fits in 8.
+__device__ __forceinline__ float below_bf16(float x) {
+  return x - __uint_as_float(__float_as_uint(x) & 0xFFFF0000u);
+}
+__device__ __forceinline__ uint32_t upper_halves(float x, float y) {
+  return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
 }
 
 // One unit of a warp's work: rows c0 .. c0 + CH - 1 of the set of one item
@@ -110,7 +125,7 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
   }
   const uint32_t ring = ((smem_u32(smem_raw) + 1023u) & ~1023u) + warp * C::kWarpBytes;
   const uint32_t qbuf = ring + kRgStages * kRgTile;
-  const float sl2 = rsqrtf(float(D)) * 1.4426950408889634f;   // scale * log2(e)
+  constexpr float sl2 = float((D == 64 ? 0.125 : 0.08838834764831844) * 1.4426950408889634);   // log2(e) / sqrt(d)
 
   // items v * n_bh + bh, from the warp's index on in steps of the grid's warps: the
   // warps at work spread over the heads, so their hot rows spread over the L2
@@ -206,7 +221,7 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
     for (int i = 0; i < QV; ++i) {
       const int e = i * 32 + lane, c = e % C::kLpr;
       int h = e / C::kLpr;
-      if (PF == kProbSplitCols) h &= 3;   // columns 4..7 repeat the heads
+      if (PF == kProbCols1 || PF == kProbCols2 || PF == kProbCols4) h &= PF - 1;   // repeated heads
       qn[i] = make_uint4(0u, 0u, 0u, 0u);
       if (h < G)
         qn[i] = __ldg(reinterpret_cast<const uint4*>(
@@ -334,20 +349,23 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
     const bool last = !MULTI || cur.c0 + CH >= cur.n;   // the item's last unit
     if (last && nxt.bh >= 0) load_q(nxt);
     // ---- softmax over the rows of each column (columns 2t and 2t + 1 in this thread)
-    uint32_t ph[NT][MT][2], pl[PF == kProbSplitMma ? NT : 1][PF == kProbSplitMma ? MT : 1][2];
+    constexpr int NP = PF == kProbMma3 ? 3 : PF == kProbCols4 ? 2 : 1;   // MMAs of a step
+    uint32_t pr[NP][NT][MT][2];
+    const uint32_t part_mask = t == 0 ? 0xFFFFFFFFu : t == 1 ? 0xFFFFu : 0u;   // kProbCols1
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       float x0 = -INFINITY, x1 = -INFINITY;
 #pragma unroll
       for (int mt = 0; mt < MT; ++mt) {
         x0 = fmaxf(x0, fmaxf(s[nt][mt][0], s[nt][mt][2]));
-        x1 = fmaxf(x1, fmaxf(s[nt][mt][1], s[nt][mt][3]));
+        if (PF != kProbCols1) x1 = fmaxf(x1, fmaxf(s[nt][mt][1], s[nt][mt][3]));
       }
 #pragma unroll
       for (int w = 4; w < 32; w <<= 1) {
         x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, w));
-        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, w));
+        if (PF != kProbCols1) x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, w));
       }
+      if (PF == kProbCols1) x1 = x0;
       x0 *= sl2;
       x1 *= sl2;
       if (MULTI) {
@@ -373,21 +391,48 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
 #pragma unroll
         for (int half = 0; half < 2; ++half) {   // rows g and g + 8
           const float p0 = ex2_fast(fmaf(s[nt][mt][2 * half], sl2, -x0));
-          const float p1 = ex2_fast(fmaf(s[nt][mt][2 * half + 1], sl2, -x1));
-          uint32_t hi = pack_bf16(p0, p1);
-          if (PF != kProbBf16) {
-            const uint32_t lo = pack_bf16(p0 - __uint_as_float(hi << 16),
-                                          p1 - __uint_as_float(hi & 0xFFFF0000u));
-            if (PF == kProbSplitCols) {
-              if (t >= 2) hi = lo;   // columns 4..7 repeat the heads with the low parts
-            } else {
-              pl[nt][mt][half] = movm_t(lo);
-            }
+          if (PF == kProbCols1) {   // every column is the head: hi, mid and lo in columns 0, 1 and 2
+            const float r = below_bf16(p0), lo = below_bf16(r);
+            pr[0][nt][mt][half] = movm_t(upper_halves(t == 0 ? p0 : lo, r) & part_mask);
+            continue;
           }
-          ph[nt][mt][half] = movm_t(hi);
+          const float p1 = ex2_fast(fmaf(s[nt][mt][2 * half + 1], sl2, -x1));
+          if (PF == kProbBf16) {
+            pr[0][nt][mt][half] = movm_t(pack_bf16(p0, p1));
+            continue;
+          }
+          if (NP > 1) {   // this lane's rows of the columns' sums
+            l[nt][0] += p0;
+            l[nt][1] += p1;
+          }
+          const float r0 = below_bf16(p0), r1 = below_bf16(p1);
+          const uint32_t hi = upper_halves(p0, p1), mid = upper_halves(r0, r1);
+          const uint32_t lo = upper_halves(below_bf16(r0), below_bf16(r1));
+          if (PF == kProbCols2) {   // columns 2t, 2t + 1: part t of the heads (part 3: zero)
+            pr[0][nt][mt][half] = movm_t(t == 0 ? hi : t == 1 ? mid : t == 2 ? lo : 0u);
+          } else if (PF == kProbCols4) {   // columns 4..7: the heads' middle parts
+            pr[0][nt][mt][half] = movm_t(t < 2 ? hi : mid);
+            pr[NP - 1][nt][mt][half] = movm_t(t < 2 ? lo : 0u);
+          } else {
+            pr[0][nt][mt][half] = movm_t(hi);
+            pr[NP / 2][nt][mt][half] = movm_t(mid);
+            pr[NP - 1][nt][mt][half] = movm_t(lo);
+          }
         }
     }
-    // ---- O^T += V_rows^T P^T, and the row sums of the same probabilities from a row of ones
+    // acc += rows^T P^T of step mt; the smaller parts are summed first, so that a step rounds the
+    // accumulator twice at most
+    auto add_parts = [&](float (&acc)[4], uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, int nt, int mt) {
+      if (NP > 1) {
+        float e[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int n = NP - 1; n > 0; --n) mma_bf16(e, x0, x1, x2, x3, pr[n][nt][mt][0], pr[n][nt][mt][1]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] += e[k];
+      }
+      mma_bf16(acc, x0, x1, x2, x3, pr[0][nt][mt][0], pr[0][nt][mt][1]);
+    };
+    // ---- O^T += V_rows^T P^T, and, of single MMAs, the row sums from a row of ones
 #pragma unroll
     for (int ti = 0; ti < TPC; ++ti) {
       cp_async_wait_group<kRgStages - 1>();
@@ -402,19 +447,13 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
                       (i >> 2) * 128,
                   x);
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            mma_bf16(o[nt][i], x[0], x[1], x[2], x[3], ph[nt][mt][0], ph[nt][mt][1]);
-            if (PF == kProbSplitMma)
-              mma_bf16(o[nt][i], x[0], x[1], x[2], x[3], pl[nt][mt][0], pl[nt][mt][1]);
-          }
+          for (int nt = 0; nt < NT; ++nt)
+            add_parts(o[nt][i], x[0], x[1], x[2], x[3], nt, mt);
         }
         constexpr uint32_t kOnes = 0x3F803F80u;
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          mma_bf16(l[nt], kOnes, kOnes, kOnes, kOnes, ph[nt][mt][0], ph[nt][mt][1]);
-          if (PF == kProbSplitMma)
-            mma_bf16(l[nt], kOnes, kOnes, kOnes, kOnes, pl[nt][mt][0], pl[nt][mt][1]);
-        }
+        for (int nt = 0; nt < NT; ++nt)
+          if (NP == 1) mma_bf16(l[nt], kOnes, kOnes, kOnes, kOnes, pr[0][nt][mt][0], pr[0][nt][mt][1]);
       }
       copy_ahead(TPC + ti);
     }
@@ -422,14 +461,33 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
     if (last) {
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
-        if (PF == kProbSplitCols) {   // columns c and c + 4 are one head's high and low parts
+        // the parts of a head in other columns
+        auto join = [](float& a, float& b) {   // columns 2t and 2t + 1 of a row
+          if (PF == kProbCols1) {   // 0, 1, 2 and 3
+            a += b;
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+          } else if (PF == kProbCols2) {   // 2t and 2t + 1, for every t
+            a += __shfl_xor_sync(0xffffffffu, a, 1);
+            b += __shfl_xor_sync(0xffffffffu, b, 1);
+          }
+          if (PF == kProbCols2 || PF == kProbCols4) {   // c and c + 4
+            a += __shfl_xor_sync(0xffffffffu, a, 2);
+            b += __shfl_xor_sync(0xffffffffu, b, 2);
+          }
+        };
 #pragma unroll
-          for (int i = 0; i < DT; ++i)
+        for (int i = 0; i < DT; ++i) {
+          join(o[nt][i][0], o[nt][i][1]);
+          join(o[nt][i][2], o[nt][i][3]);
+        }
+        if (NP == 1) {
+          join(l[nt][0], l[nt][1]);
+        } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-              o[nt][i][e] += __shfl_xor_sync(0xffffffffu, o[nt][i][e], 2);
-          l[nt][0] += __shfl_xor_sync(0xffffffffu, l[nt][0], 2);
-          l[nt][1] += __shfl_xor_sync(0xffffffffu, l[nt][1], 2);
+          for (int w = 4; w < 32; w <<= 1) {
+            l[nt][0] += __shfl_xor_sync(0xffffffffu, l[nt][0], w);
+            l[nt][1] += __shfl_xor_sync(0xffffffffu, l[nt][1], w);
+          }
         }
         const float i0 = 1.f / l[nt][0], i1 = 1.f / l[nt][1];
 #pragma unroll
@@ -499,18 +557,22 @@ template <int D>
 cudaError_t launch_gather_d(const ReplayArgs& a, int num_sms, cudaStream_t st) {
   const int G = a.d.Hq / a.d.Hkv;
   if (a.full || a.d.S > 128)
-    return G <= 4   ? launch_gather_multi<D, 1, kProbSplitCols>(a, num_sms, st)
-           : G <= 8 ? launch_gather_multi<D, 1, kProbSplitMma>(a, num_sms, st)
-                    : launch_gather_multi<D, 2, kProbSplitMma>(a, num_sms, st);
+    return G == 1   ? launch_gather_multi<D, 1, kProbCols1>(a, num_sms, st)
+           : G == 2 ? launch_gather_multi<D, 1, kProbCols2>(a, num_sms, st)
+           : G <= 4 ? launch_gather_multi<D, 1, kProbCols4>(a, num_sms, st)
+           : G <= 8 ? launch_gather_multi<D, 1, kProbMma3>(a, num_sms, st)
+                    : launch_gather_multi<D, 2, kProbMma3>(a, num_sms, st);
   // d = 128 sets of at most 128 rows take bf16 probabilities, like the full-attention
-  // kernel; everything else keeps fp32 probabilities as hi + lo
+  // kernel; everything else keeps fp32 probabilities in three parts
   if constexpr (D == 128)
     return G <= 8 ? launch_gather_one<D, 1, kProbBf16>(a, num_sms, st)
                   : launch_gather_one<D, 2, kProbBf16>(a, num_sms, st);
   else
-    return G <= 4   ? launch_gather_one<D, 1, kProbSplitCols>(a, num_sms, st)
-           : G <= 8 ? launch_gather_one<D, 1, kProbSplitMma>(a, num_sms, st)
-                    : launch_gather_one<D, 2, kProbSplitMma>(a, num_sms, st);
+    return G == 1   ? launch_gather_one<D, 1, kProbCols1>(a, num_sms, st)
+           : G == 2 ? launch_gather_one<D, 1, kProbCols2>(a, num_sms, st)
+           : G <= 4 ? launch_gather_one<D, 1, kProbCols4>(a, num_sms, st)
+           : G <= 8 ? launch_gather_one<D, 1, kProbMma3>(a, num_sms, st)
+                    : launch_gather_one<D, 2, kProbMma3>(a, num_sms, st);
 }
 
 }  // namespace

@@ -366,3 +366,40 @@ def test_selection_bounds_lists_and_fallback(max_seq, top_s):
             ref = np.sort(np.lexsort((np.arange(u + 1), -key))[:top_s])
             np.testing.assert_array_equal(sel[b, u, :ref.size], ref, err_msg=f"b={b} u={u}")
             assert (sel[b, u, ref.size:] == -1).all()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("group,top_s,n", [(1, 128, 99), (2, 64, 63), (4, 128, 99), (6, 128, 99), (16, 128, 99),
+                                           (1, 256, 201), (2, 256, 201), (3, 256, 201), (7, 256, 201),
+                                           (12, 256, 201)])
+def test_probabilities_keep_fp32(d, group, top_s, n):
+    """Values +1 and -1 on neighbouring keys that score almost alike: what is left of the weights is
+    about 1e-5, so an error of the weights shows. Sets of more than 128 rows, sets of 64-wide heads
+    and full layers of a context that is not a multiple of 8 keep fp32 weights. With n keys of weight
+    1 / n, fp32 weights are off by about 2^-24 / sqrt(n) (rms) and a sum of two bf16 by 2^-18.8 /
+    sqrt(n), which is 2.2e-7 at n = 99; the bound is 2^-24 beside the output's own rounding (2^-9)."""
+    import _helpers as H
+    wl = RW("r_cancel", 2, 3, group, 1, d, 1, n, (n,), top_s=top_s, n_full=1)
+    rng = np.random.default_rng(group + n)
+    q = rng.standard_normal((1, group, n, d)).astype(np.float32)
+    k = rng.standard_normal((1, 1, n, d)).astype(np.float32) * 0.25
+    k[:, :, 1::2] = k[:, :, 0:n - 1:2]
+    q[..., 0] *= 2.0 ** -10
+    k[:, :, 1::2, 0] += 0.25
+    v = np.ones((1, 1, n, d), np.float32)
+    v[:, :, 1::2] = -1.0
+    v *= 1.0 + np.arange(d, dtype=np.float32) / 64 % 1
+    bits = [H.f32_to_bf16_bits(x) for x in (q, k, v)]
+    g = synth.gen_guide(wl, 3)
+    run = ReplayRun(wl)
+    us = np.arange(31, n, 2)   # whole pairs of keys
+    for layer in (0, 1) if d == 64 or top_s > 128 else (0,):   # 0: full; 1: guided, over 0..u (u < top_s)
+        got = _f64(run.attend(layer, *bits, None if layer == 0 else g))[0][:, us]
+        qd, kd, vd = (H.bf16_bits_to_f64(x)[0] for x in bits)
+        s = np.einsum("hud,jd->huj", qd[:, us], kd[0]) / np.sqrt(d)
+        s[:, np.arange(n)[None] > us[:, None]] = -np.inf
+        p = np.exp(s - s.max(2, keepdims=True))
+        ref = np.einsum("huj,jd->hud", p / p.sum(2, keepdims=True), vd[0])
+        rms = lambda x: float(np.sqrt(np.mean(x * x)))
+        assert 1e-6 < rms(ref) < 1e-4
+        assert rms(got - ref) <= 2.0 ** -9 * rms(ref) + 2.0 ** -24, (layer, rms(got - ref), rms(ref))
