@@ -86,6 +86,64 @@ __device__ __forceinline__ uint32_t upper_halves(float x, float y) {
   return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
 }
 
+// Two bf16 each: acc + 0 w, which is NaN from the first infinity or NaN on.
+__device__ __forceinline__ uint32_t zero_times(uint32_t w, uint32_t acc) {
+  uint32_t r;
+  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(0u), "r"(acc));
+  return r;
+}
+
+// The values of an item that came out infinite or NaN, again: one warp, key by key in fp32. In the
+// MMAs an infinite value row also meets the probability 0 of the slots that fill up a unit, and
+// the small parts of its own probability, which may be 0: infinity times 0 is NaN. Here it meets
+// its own probability alone. Everything finite stays.
+template <int D>
+__device__ __noinline__ void redo_non_finite(const ReplayArgs& a, int bh, int u, int n, const int32_t* sel) {
+  constexpr int DL = D / 32;   // dimensions per lane
+  const ReplayDims& d = a.d;
+  const int lane = threadIdx.x & 31, G = d.Hq / d.Hkv;
+  const float scale = rsqrtf(float(D));
+  const uint16_t* kb = static_cast<const uint16_t*>(a.k) + int64_t(bh) * d.N * D;
+  const uint16_t* vb = static_cast<const uint16_t*>(a.v) + int64_t(bh) * d.N * D;
+  for (int h = 0; h < G; ++h) {
+    const int64_t at = ((int64_t(bh) * G + h) * d.N + u) * D;
+    const uint16_t* qr = static_cast<const uint16_t*>(a.q) + at;
+    auto key = [&](int j) { return sel == nullptr ? j : sel[j]; };
+    auto score = [&](int row) {
+      const uint16_t* kr = kb + int64_t(row) * D;
+      float x = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < D; ++c) x = fmaf(bf16f(qr[c]) * scale, bf16f(kr[c]), x);
+      return x;
+    };
+    float m = -INFINITY, l = 0.f, o[DL];
+#pragma unroll 1
+    for (int j = lane; j < n; j += 32) m = fmaxf(m, score(key(j)));
+    for (int w = 16; w > 0; w >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, w));
+#pragma unroll
+    for (int e = 0; e < DL; ++e) o[e] = 0.f;
+#pragma unroll 1
+    for (int j0 = 0; j0 < n; j0 += 32) {
+      const bool in = j0 + lane < n;
+      const int row = in ? key(j0 + lane) : 0;
+      const float p = in ? expf(score(row) - m) : 0.f;
+      l += p;
+#pragma unroll 1
+      for (int i = 0; i < min(32, n - j0); ++i) {
+        const float pi = __shfl_sync(0xffffffffu, p, i);
+        const uint16_t* vr = vb + int64_t(__shfl_sync(0xffffffffu, row, i)) * D + lane * DL;
+#pragma unroll
+        for (int e = 0; e < DL; ++e) o[e] = fmaf(pi, bf16f(vr[e]), o[e]);
+      }
+    }
+    for (int w = 16; w > 0; w >>= 1) l += __shfl_xor_sync(0xffffffffu, l, w);
+    uint16_t* out = static_cast<uint16_t*>(a.out) + at + lane * DL;
+#pragma unroll
+    for (int e = 0; e < DL; ++e)
+      if ((out[e] & 0x7F80u) == 0x7F80u) out[e] = __bfloat16_as_ushort(__float2bfloat16_rn(o[e] / l));
+  }
+}
+
 // One unit of a warp's work: rows c0 .. c0 + CH - 1 of the set of one item
 // (bh = b * Hkv + hk, position u); bh < 0 past the last item.
 struct Unit {
@@ -501,13 +559,20 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
         }
       }
       __syncwarp();
+      uint32_t odd = 0u;   // NaN where a value is not finite
 #pragma unroll
       for (int i = 0; i < QV; ++i) {
         const int e = i * 32 + lane, h = e / C::kLpr, c = e % C::kLpr;
-        if (h < G)
+        if (h < G) {
+          const uint4 w = ld_shared_v4(qbuf + h * C::kRow + ((((c & 7) ^ (h & 7)) | (c & ~7)) << 4));
           *reinterpret_cast<uint4*>(static_cast<uint16_t*>(a.out) +
-                                    ((int64_t(cur.bh) * G + h) * d.N + cur.u) * D + 8 * c) =
-              ld_shared_v4(qbuf + h * C::kRow + ((((c & 7) ^ (h & 7)) | (c & ~7)) << 4));
+                                    ((int64_t(cur.bh) * G + h) * d.N + cur.u) * D + 8 * c) = w;
+          odd = zero_times(w.w, zero_times(w.z, zero_times(w.y, zero_times(w.x, odd))));
+        }
+      }
+      if (__any_sync(0xffffffffu, odd != 0u)) {
+        __syncwarp();
+        redo_non_finite<D>(a, cur.bh, cur.u, FULL ? cur.u + 1 : cur.n, FULL ? nullptr : sel_c - cur.c0 - 8 * grp);
       }
     }
     cur = nxt;

@@ -403,3 +403,60 @@ def test_probabilities_keep_fp32(d, group, top_s, n):
         rms = lambda x: float(np.sqrt(np.mean(x * x)))
         assert 1e-6 < rms(ref) < 1e-4
         assert rms(got - ref) <= 2.0 ** -9 * rms(ref) + 2.0 ** -24, (layer, rms(got - ref), rms(ref))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("group,top_s,n", [(1, 100, 131), (2, 40, 67), (4, 200, 261), (6, 128, 195), (12, 130, 197)])
+def test_infinities_and_nans(d, group, top_s, n):
+    """An infinity in a value row makes infinite what takes the row with a positive weight, in its
+    dimension, and nothing else; a key whose score is -inf takes no part, also where whole units of
+    keys score -inf; +inf and NaN scores, and infinities of both signs, give NaN. Every query of a
+    full layer (n not a multiple of 8) and of a guided layer against the same in numpy."""
+    import _helpers as H
+    wl = RW("r_inf", 2, 3, group, 1, d, 1, n, (n,), top_s=top_s, n_full=1)
+    q, k, v = synth.gen_replay_qkv(wl, 43)
+    g = synth.gen_guide(wl, 47)
+    q[..., 0] &= 0x7FFF
+    q[..., 1] &= 0x7FFF
+    q[0, 0, n - 2:, 1] |= 0x8000       # one head's last queries meet k = -inf with a negative q
+    run = ReplayRun(wl)
+    sel = run.select(g)[0]
+    cases = []
+    k1, v1 = k.copy(), v.copy()
+    v1[0, 0, [3, 60], 17] = 0x7F80     # +inf
+    v1[0, 0, n // 2, 18] = 0xFF80      # -inf
+    v1[0, 0, 5, 19], v1[0, 0, 9, 19] = 0x7F80, 0xFF80
+    v1[0, 0, 20, 20] = 0x7FC0
+    cases.append((k1, v1))
+    k2, v2 = k.copy(), v.copy()
+    k2[0, 0, 1:70, 0] = 0xFF80         # score -inf: more than the first unit of 64 but one key
+    k2[0, 0, n - 1, 1] = 0xFF80
+    cases.append((k2, v2))
+    k3 = k2.copy()
+    k3[0, 0, 0, 0] = 0xFF80            # the whole first unit
+    cases.append((k3, v2))
+    for layer in (0, 1):
+        clean = run.attend(layer, q, k, v, None if layer == 0 else g).cpu().numpy()[0]
+        for kk, vv in cases:
+            out = run.attend(layer, q, kk, vv, None if layer == 0 else g)
+            got, raw = _f64(out)[0], out.cpu().numpy()[0]
+            qd, kd, vd = (H.bf16_bits_to_f64(x)[0] for x in (q, kk, vv))
+            with np.errstate(invalid="ignore", over="ignore"):
+                s = np.einsum("hud,jd->huj", qd, np.where(np.isinf(kd[0]), 0, kd[0])) / np.sqrt(d)
+                for j, c in zip(*np.nonzero(np.isinf(kd[0]))):
+                    s[:, :, j] += qd[:, :, c] * kd[0, j, c]
+                for u in range(n):
+                    at = np.arange(u + 1) if layer == 0 else sel[u][sel[u] >= 0]
+                    p = np.exp(s[:, u, at] - s[:, u, at].max(1, keepdims=True))
+                    ref = (p / p.sum(1, keepdims=True)) @ np.where(np.isfinite(vd[0, at]), vd[0, at], 0)
+                    for i, c in zip(*np.nonzero(~np.isfinite(vd[0, at]))):
+                        ref[:, c] += np.where(p[:, i] > 0, 1.0, np.nan) * vd[0, at[i], c]
+                    x = got[:, u]
+                    assert (np.isnan(x) == np.isnan(ref)).all(), u
+                    assert (x[np.isinf(ref)] == ref[np.isinf(ref)]).all(), u
+                    fin = np.isfinite(ref)
+                    assert np.isfinite(x[fin]).all(), u
+                    if kk is k1:       # scores as before: what is finite has the clean run's bits
+                        assert (raw[:, u][fin] == clean[:, u][fin]).all(), u
+                    elif fin.any():
+                        G.assert_parity(BF16, x[fin], ref[fin], f"layer {layer} u {u}")
