@@ -116,7 +116,9 @@ __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* p) {
 //
 // pdl_enter: let the next kernel of the stream start its prologue as SMs come free, and wait
 // until the kernel before this one (if this launch may overlap it) has finished and its writes
-// are visible. Everything before it touches nothing that another kernel writes.
+// are visible. Everything before it touches nothing that another kernel of the call writes. Every
+// CTA calls it, also one without work: a grid whose CTAs all leave without waiting may be complete
+// before its predecessor is, and the next call is ordered behind that grid alone.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

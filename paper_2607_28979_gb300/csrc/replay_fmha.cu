@@ -221,9 +221,12 @@ __global__ void __launch_bounds__(Fa<D>::kThreads, 1)
   const int bh = static_cast<int>(blockIdx.x / n_qt);
   const int b = bh / d.Hq, h = bh - b * d.Hq;
   const int hk = h / (d.Hq / d.Hkv);
-  const int L = seq_len_of(a, b);
+  const int L = seq_len_of(a, b);   // an input of the call: the kernel before this one does not write it
   const int q0 = qt * 128;
-  if (q0 >= L) return;   // uniform over the CTA: no barrier or TMEM use yet
+  if (q0 >= L) {   // uniform over the CTA: no barrier or TMEM use yet
+    pdl_enter();
+    return;
+  }
   const int n_kv = qt + 1;
   const long long wl = a.wait_limit;
 

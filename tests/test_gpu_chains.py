@@ -109,3 +109,26 @@ def test_chain_captured_and_back_to_back(name):
     for i, o in got:
         assert all(bool((a == b).all()) for a, b in zip(o, want[i]))
     assert name.startswith("replay") or M.mot_get_device_status(h) == M.MOT_OK
+
+
+def test_a_full_layer_behind_an_empty_one():
+    """A full-attention call whose sequences are all empty, directly followed by an ordinary one on the
+    same handle: the second transposes V into the workspace that the first's transpose still writes if
+    the first's attention grid is complete too early."""
+    wl = SHAPES["replay_full"][0].replace(max_seq=2048, seq_lens=(2048, 1300))
+    h = M.mot_create_replay(M.replay_config_from(wl))
+    lens = torch.tensor(wl.seq_lens, dtype=torch.int32, device="cuda")
+    none = torch.zeros_like(lens)
+    a, b = [[_bf16(x) for x in synth.gen_replay_qkv(wl, s)] for s in (1, 2)]
+    want = torch.zeros(wl.max_batch, wl.q_heads, wl.max_seq, wl.head_dim, dtype=torch.int16, device="cuda")
+    M.mot_replay_attention(h, 0, *b, None, lens, 2, want)
+    torch.cuda.synchronize()
+    outs = [torch.zeros_like(want) for _ in range(20)]
+    untouched = torch.full_like(want, 7)
+    for o in outs:
+        M.mot_replay_attention(h, 0, *a, None, none, 2, untouched)
+        M.mot_replay_attention(h, 0, *b, None, lens, 2, o)
+    torch.cuda.synchronize()
+    assert bool((untouched == 7).all()) and bool((want != 0).any())
+    for o in outs:
+        assert torch.equal(o, want)
