@@ -410,7 +410,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         uint4 bias[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) bias[i] = __ldg(bias4 + j * (kChunk / 8) + i);
-        const float gate = valid ? __ldg(grow + (j * kChunk) / d.H) : 0.f;
+        const float gate = valid ? ld_chain(grow + (j * kChunk) / d.H) : 0.f;
         int w = 1;
         if (lane == 0) w = mbar_wait(&bars->a1full[b], (c >> 1) & 1u, abort_flag, p.wait_limit);
         if (!__shfl_sync(0xffffffffu, w, 0)) { ok = false; break; }

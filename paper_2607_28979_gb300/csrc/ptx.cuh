@@ -124,6 +124,22 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// What the kernel before this one wrote: a coherent load, behind pdl_enter. __ldg's non-coherent one
+// is for data that nothing writes while the kernel is resident (weights, the caller's inputs), and
+// this kernel may be resident while its predecessor writes.
+__device__ __forceinline__ float ld_chain(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int4 ld_chain(const int4* p) {
+  int4 v;
+  asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
 // ---------------------------------------------------------------- cp.async (16-byte copies)
 
 // One 16-byte global -> shared copy (L2 only, not L1), tracked by commit groups.

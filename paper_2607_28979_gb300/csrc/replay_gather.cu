@@ -252,8 +252,8 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
       for (int i = 0; i < 8; ++i) idx[i] = min(w.c0 + tr * C::kRows + 8 * grp + i, w.n - 1);
     } else if (w.bh >= 0) {
       const int off = (tr * C::kRows + rot) & (CH - 1);
-      const int4 x = __ldg(reinterpret_cast<const int4*>(sel + off));
-      const int4 y = __ldg(reinterpret_cast<const int4*>(sel + off + 4));
+      const int4 x = ld_chain(reinterpret_cast<const int4*>(sel + off));
+      const int4 y = ld_chain(reinterpret_cast<const int4*>(sel + off + 4));
       idx[0] = x.x; idx[1] = x.y; idx[2] = x.z; idx[3] = x.w;
       idx[4] = y.x; idx[5] = y.y; idx[6] = y.z; idx[7] = y.w;
     }

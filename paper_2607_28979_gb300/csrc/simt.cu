@@ -43,6 +43,8 @@ __device__ __forceinline__ float ld_f(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float ld_f(const __nv_bfloat16* p) {
   return __bfloat162float(__ushort_as_bfloat16(__ldg(reinterpret_cast<const uint16_t*>(p))));
 }
+__device__ __forceinline__ float ld_a2(const float* p) { return ld_chain(p); }   // GEMM1 writes it
+__device__ __forceinline__ float ld_a2(const __nv_bfloat16*) { return 0.f; }      // never: a2 is fp32
 __device__ __forceinline__ void st_v(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st_v(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
           const TA* src = GEMM == 1
                               ? abase + (static_cast<size_t>(h) * d.S + r) * d.d_s + (cc - h * d.d_s)
                               : abase + static_cast<size_t>(r) * d.EH + cc;
-          dst[e] = r < nrows && cc < K ? ld_f(src) : 0.f;
+          dst[e] = r < nrows && cc < K ? (GEMM == 1 ? ld_f(src) : ld_a2(src)) : 0.f;
         }
       }
     }

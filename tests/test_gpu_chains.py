@@ -20,6 +20,7 @@ SHAPES = {
     "pair": (W("c_pair", 3, 2, 64, 4, 2, 128, 2, 256, 4, 300, "bf16", (300, 129, 1)), M.SCHEDULE_PAIR),
     "onchip": (W("c_onchip", 2, 2, 64, 3, 2, 128, 3, 256, 2, 64, "bf16", (64, 33)), M.SCHEDULE_ONCHIP),
     "fp32": (W("c_fp32", 3, 2, 12, 2, 3, 10, 2, 50, 3, 90, "fp32", (90, 0, 65)), None),
+    "fp32_scalar": (W("c_fp32s", 3, 2, 12, 2, 3, 10, 3, 33, 3, 90, "fp32", (90, 0, 65)), None),
     "routed": (W("c_routed", 2, 2, 64, 2, 2, 128, 4, 256, 2, 160, "bf16", (160, 33), top_k=2), None),
     "activations": (W("c_h", 3, 1, 128, 3, 2, 128, 3, 256, 2, 130, "bf16", (130, 7), act_tgt=256), None),
     "backbones": (W("c_bt", 3, 5, 64, 5, 3, 32, 2, 0, 2, 29, "bf16", (29, 14), top_k=1,

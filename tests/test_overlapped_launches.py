@@ -48,3 +48,12 @@ def test_every_cta_of_an_overlapped_kernel_waits_before_it_leaves():
         wait = body.find("pdl_enter();")
         assert wait >= 0, name
         assert not re.search(r"\breturn\b\s*;", body[:wait]), name
+
+
+def test_workspaces_of_a_chain_are_not_read_through_the_non_coherent_path():
+    """__ldg wants data that nothing writes while the kernel is resident; an overlapped kernel is
+    resident while its predecessor writes the gate rows, the hidden rows and the selection."""
+    kernels = _kernels()
+    for name in _overlapped():
+        for m in re.finditer(r"__ldg\(([^;]*)", kernels[name]):
+            assert not re.search(r"\b(sel|grow|a2|tiles|n_tiles|rvt)\b|\.gate\b", m.group(1)), (name, m.group(0)[:80])
