@@ -1385,13 +1385,8 @@ cudaError_t launch_bt_gate(const BtArgs& a, cudaStream_t st) {
   const size_t smem = size_t(d.E) * d.N * d.Ds * 2;
   const int em = d.E <= 2 ? 0 : d.E <= 4 ? 1 : 2;
   auto kern = em == 0 ? bt_gate_kernel<2> : em == 1 ? bt_gate_kernel<4> : bt_gate_kernel<8>;
-  static size_t attr[3] = {0, 0, 0};
-  if (smem > 48 * 1024 && smem > attr[em]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    attr[em] = smem;
-  }
+  static SmemOptIn opt_in[3];
+  if (cudaError_t e = opt_in[em](kern, static_cast<int>(smem))) return e;
   const int n_tok = d.B * d.S;
   dim3 grid(std::min((n_tok + 15) / 16, 1024), 2);
   kern<<<grid, 256, smem, st>>>(a);
@@ -1422,10 +1417,8 @@ cudaError_t launch_bt_attn(const BtArgs& a, cudaStream_t st) {
   const int max_tok = (256 / d.na + 2) / d.P + 2;
   const int smem = max_tok * d.P * 2 * d.d * 2;
   auto kern = d.d / d.na == 16 ? bt_attn_kernel<16> : d.d / d.na == 32 ? bt_attn_kernel<32> : bt_attn_kernel<64>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-  }
+  static SmemOptIn opt_in[3];
+  if (cudaError_t e = opt_in[d.d / d.na == 16 ? 0 : d.d / d.na == 32 ? 1 : 2](kern, smem)) return e;
   kern<<<grid, 256, smem, st>>>(a);
   return cudaGetLastError();
 }
@@ -1472,16 +1465,11 @@ cudaError_t launch_bt_gemm(int mode, const BtArgs& a, const CUtensorMap& tmA,
   if (c.NT < 32 || c.NT > 256 || c.NT % 32 || c.K % 64) return cudaErrorInvalidValue;
   // the row-norm stages keep a row in one thread; the others spread it over 16 warps
   const bool wide = mode == kBtQ || mode == kBtKV || mode == kBtF1 || mode == kBtOut;
-  static bool attr_set[4] = {false, false, false, false};
+  static SmemOptIn opt_in[4];
   const int di = (d.d == 128 ? 1 : 0) + (wide ? 2 : 0);
   auto kern = wide ? (d.d == 128 ? bt_gemm_kernel<128, 16> : bt_gemm_kernel<64, 16>)
                    : (d.d == 128 ? bt_gemm_kernel<128, kBtRowEpi> : bt_gemm_kernel<64, kBtRowEpi>);
-  if (!attr_set[di]) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBtSmem);
-    if (e != cudaSuccess) return e;
-    attr_set[di] = true;
-  }
+  if (cudaError_t e = opt_in[di](kern, kBtSmem)) return e;
   const long long items =
       static_cast<long long>(c.groups) * c.row_tiles * c.n_tiles * std::max(c.slots, 1);
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
@@ -1501,15 +1489,10 @@ cudaError_t launch_bt_ffn(const BtArgs& a, const CUtensorMap& tmXf, const CUtens
   c.n_tiles = 1;
   c.NT = d.d;
   c.K = d.df;
-  static bool attr[2] = {false, false};
-  const int di = d.d == 128 ? 1 : 0;
+  static SmemOptIn opt_in[2];
   auto kern = d.d == 128 ? bt_ffn_kernel<128> : bt_ffn_kernel<64>;
   const int smem = d.d == 128 ? Ffn<128>::kSmem : Ffn<64>::kSmem;
-  if (!attr[di]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr[di] = true;
-  }
+  if (cudaError_t e = opt_in[d.d == 128 ? 1 : 0](kern, smem)) return e;
   const long long items = static_cast<long long>(c.groups) * c.row_tiles;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
   if (grid <= 0) return cudaSuccess;

@@ -898,13 +898,8 @@ cudaError_t launch_scan(const BtArgs& a, const CUtensorMap (&tm)[6], int num_sms
   c.row_tiles = d.B * d.tiles_b;
   c.n_tiles = 1;
   auto kern = bt_scan_kernel<NXV, DH>;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kScMaxSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(kern, kScMaxSmem)) return e;
   const int n_ring = ring_blocks(d.df), at = ring_off(d.df);
   const long long items = static_cast<long long>(c.groups) * c.row_tiles;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);

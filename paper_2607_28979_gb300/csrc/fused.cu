@@ -340,13 +340,8 @@ cudaError_t launch_fused(const PathArgs& a, const CUtensorMap& tmK, const CUtens
                          const CUtensorMap& tmW2, const CUtensorMap& tmA2st,
                          const CUtensorMap& tmG16, const CUtensorMap& tmB2t, int32_t* counters,
                          int num_sms, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(mot_fused_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(mot_fused_kernel, kSmemBytes)) return e;
   cudaError_t e = cudaMemsetAsync(counters, 0, fused_counter_ints(a.d, a.gp) * sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   FusedArgs fa;

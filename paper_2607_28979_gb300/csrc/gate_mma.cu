@@ -276,13 +276,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
 
 cudaError_t launch_gate_mma(const PathArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV,
                             const CUtensorMap& tmWg, int num_sms, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(gate_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(gate_mma_kernel, kGSmem)) return e;
   const long long items = static_cast<long long>(a.gp) * a.d.tiles_max;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);
   if (grid <= 0) return cudaSuccess;

@@ -8,6 +8,7 @@
 #include <utility>
 
 #include "mot.h"
+#include "smem_opt_in.h"
 
 #include <nvtx3/nvToolsExt.h>
 

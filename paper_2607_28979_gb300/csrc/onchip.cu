@@ -531,13 +531,8 @@ cudaError_t launch_onchip(const PathArgs& a, const CUtensorMap& tmK, const CUten
                           const CUtensorMap& tmW1q, const CUtensorMap& tmW2h,
                           const CUtensorMap& tmG16, const CUtensorMap& tmB2th, int num_sms,
                           cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(onchip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(onchip_kernel, kSmemBytes)) return e;
   OnchipArgs oa;
   oa.p = a;
   oa.nk1 = a.d.Ds / UK;

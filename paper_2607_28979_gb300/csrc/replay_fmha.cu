@@ -540,15 +540,10 @@ bool replay_fmha_supported(const ReplayDims& d) {
 cudaError_t launch_replay_fmha(const ReplayArgs& a, const CUtensorMap& tmK,
                                const CUtensorMap& tmVt, cudaStream_t st) {
   const ReplayDims& d = a.d;
-  static bool attr[2] = {false, false};
-  const int di = d.d == 128 ? 1 : 0;
+  static SmemOptIn opt_in[2];
   auto kern = d.d == 128 ? replay_fmha_kernel<128> : replay_fmha_kernel<64>;
   const int smem = d.d == 128 ? Fa<128>::kSmem : Fa<64>::kSmem;
-  if (!attr[di]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr[di] = true;
-  }
+  if (cudaError_t e = opt_in[d.d == 128 ? 1 : 0](kern, smem)) return e;
   const int n_qt = (d.N + 127) / 128;
   return launch_kernel(a.overlap, kern, d.B * d.Hq * n_qt, Fa<128>::kThreads, smem, st, tmK, tmVt, a);
 }

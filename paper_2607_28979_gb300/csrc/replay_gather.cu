@@ -589,13 +589,8 @@ cudaError_t launch_gather(const ReplayArgs& a, int num_sms, cudaStream_t st) {
   using C = Rg<D, NT>;
   static_assert(C::kSmem <= 232448 - 32, "shared memory budget");
   auto kernel = replay_gather_kernel<D, NT, PF, CH, MULTI, FULL>;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(kernel, C::kSmem)) return e;
   const int64_t items = int64_t(a.d.B) * a.d.Hkv * a.d.N;
   const int grid = static_cast<int>(items < num_sms ? items : num_sms);   // persistent
   return launch_kernel(a.overlap, kernel, grid, 32 * C::kWarps, C::kSmem, st, a);

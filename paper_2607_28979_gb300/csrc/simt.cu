@@ -260,13 +260,8 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_gemm_kernel(const PathAr
 template <typename T, int GEMM, bool VEC, int KS>
 cudaError_t launch_simt_v(const PathArgs& a, cudaStream_t st) {
   const Dims& d = a.d;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(simt_gemm_kernel<T, GEMM, VEC, KS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSimtSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(simt_gemm_kernel<T, GEMM, VEC, KS>, kSimtSmem)) return e;
   const int N = GEMM == 1 ? d.EH : d.Dt;
   dim3 grid(2 * d.tiles_max, (N + BN - 1) / BN, a.gp * KS);
   return launch_kernel_clusters(a.overlap, KS, simt_gemm_kernel<T, GEMM, VEC, KS>, grid, kSimtThreads,

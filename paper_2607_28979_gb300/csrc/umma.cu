@@ -262,14 +262,8 @@ template <int MODE>
 cudaError_t launch_umma(const PathArgs& a, const CUtensorMap& A0, const CUtensorMap& A1,
                         const CUtensorMap& B, const CUtensorMap& S, int nk, int n_tiles_n,
                         int b_rows, int num_sms, cudaStream_t st) {
-  static bool attr_set = false;   // per process; the attribute is per function
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(umma_gemm_kernel<MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem_bytes(MODE));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(umma_gemm_kernel<MODE>, smem_bytes(MODE))) return e;
   UmmaArgs ua;
   ua.p = a;
   ua.nk = nk;

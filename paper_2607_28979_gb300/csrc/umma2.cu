@@ -416,14 +416,8 @@ template <int MODE, bool SPARSE>
 cudaError_t launch_umma2(const PathArgs& a, const SparseArgs* sp, const CUtensorMap& A0,
                          const CUtensorMap& A1, const CUtensorMap& B, const CUtensorMap& S, int nk,
                          int n_tiles_n, int b_rows, int num_sms, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(umma2_gemm_kernel<MODE, SPARSE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem_bytes2(MODE));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(umma2_gemm_kernel<MODE, SPARSE>, smem_bytes2(MODE))) return e;
   Umma2Args ua{};
   ua.p = a;
   if (sp) ua.sp = *sp;

@@ -582,20 +582,22 @@ cudaError_t launch_wide(const PathArgs& a, const CUtensorMap& tmK, const CUtenso
                         const CUtensorMap& tmW1q, const CUtensorMap& tmW2h,
                         const CUtensorMap& tmG16, const CUtensorMap& tmB2th, int num_sms,
                         cudaStream_t st) {
-  static int max_clusters = 0;
+  static SmemOptIn smem;
+  if (cudaError_t e = smem(wide_kernel, kWSmemBytes)) return e;
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev)) return e;
+  static std::atomic<int> clusters[64] = {};   // by device
+  int max_clusters = dev < 64 ? clusters[dev].load(std::memory_order_relaxed) : 0;
   if (max_clusters == 0) {
-    cudaError_t e = cudaFuncSetAttribute(wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kWSmemBytes);
-    if (e != cudaSuccess) return e;
     // clusters that fit at once (one CTA per SM): the persistent grid's size
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(kWCtas * (num_sms / kWCtas));
     cfg.blockDim = dim3(kWThreads);
     cfg.dynamicSmemBytes = kWSmemBytes;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, wide_kernel, &cfg);
-    if (e != cudaSuccess) return e;
+    if (cudaError_t e = cudaOccupancyMaxActiveClusters(&n, wide_kernel, &cfg)) return e;
     max_clusters = n > 0 ? n : 1;
+    if (dev < 64) clusters[dev].store(max_clusters, std::memory_order_relaxed);
   }
   WideArgs wa;
   wa.p = a;
