@@ -115,6 +115,13 @@ def algorithmic_bt(wl, layer_map):
         # FFN1 + GELU + FFN2 in one kernel: no hidden rows in HBM
         "bt_ffn_fused": allrows * (d * 2 + d * 4 + d * 4 + d * 2 + d * 2 + 8),
     }
+    # the window in one launch: every slot's stages, source rows in and state rows out; then the
+    # output projections of all slots
+    per_launch["bt_scan"] = N * sum(per_launch[k] for k in ("bt_in_ln_gelu", "bt_q", "bt_kv", "bt_attn",
+                                                            "bt_o_residual_ln", "bt_ffn_fused"))
+    bpl["bt_scan"] = N * rows * (ds * es + d * 2 + 8)
+    per_launch["bt_out_all_slots"] = N * per_launch["bt_out_gelu_combine"]
+    bpl["bt_out_all_slots"] = N * (rows * (d * 2 + 8) + 2 * T * Dt * es)
     src_layers = {layer_map[t] for t in range(q, q + N)}
     bytes_src = 2 * len(src_layers) * T * Ds * es
     bytes_dst = 2 * N * T * Dt * es
@@ -175,7 +182,9 @@ KERNEL_SOURCES = {
                       "ptx.cuh"],
     "replay_fmha_full": ["replay_fmha.cu", "replay_common.cuh", "replay_internal.h",
                          "mot_internal.h", "ptx.cuh"],
-    # backbone translators (all kernels of bt.cu)
+    # backbone translators: the window's scan, and the kernels of bt.cu
+    "bt_scan": ["bt_scan.cu", "bt_common.cuh", "bt_internal.h", "gelu.cuh", "mot_internal.h",
+                "ptx.cuh"],
     "bt_ffn_fused": ["bt.cu", "bt_common.cuh", "bt_internal.h", "gelu.cuh", "mot_internal.h",
                      "ptx.cuh"],
 }
@@ -504,7 +513,7 @@ class _Setup:
             sched = "routed (Top-K token buckets)"
         if wl.is_bt:
             sched = ("backbone scan" + (" on Top-1 token buckets" if M.mot_get_routing(self.h) == 1 else "")
-                     + ", the window in one launch (the kernel list times its stages one by one)")
+                     + ", the window in one launch")
         self.schedule = sched
         self.bf = wl.dtype == "bf16"
         tdt = torch.bfloat16 if self.bf else torch.float32
@@ -544,7 +553,7 @@ def time_device(M, torch, S, args, world, rank, local):
     sampler = ClockSampler(local) if rank == 0 else None
     if sampler:
         sampler.start()
-    # a profiled backbone call runs its stages as separate kernels, so those are timed afterwards
+    # backbone calls are three or four launches: their per-kernel events are taken afterwards
     M.mot_profile_enable(S.h, not S.wl.is_bt)
     M.mot_profile_read(S.h)
     launches0 = M.mot_get_launch_count(S.h)
@@ -563,7 +572,7 @@ def time_device(M, torch, S, args, world, rank, local):
     launches = M.mot_get_launch_count(S.h) - launches0
     clocks = sampler.stop() if sampler else None
     if S.wl.is_bt:
-        M.mot_profile_enable(S.h, True)
+        M.mot_profile_enable(S.h, M.PROFILE_AS_LAUNCHED)
         for _ in range(args.steps):
             S.step()
         torch.cuda.synchronize()
@@ -726,7 +735,7 @@ def run_mot(args, wl):
                        "l2": ("inputs larger than L2 (%.2f GB read+written per step)" % (alg["bytes"] / 1e9)
                               if not wl.is_bt else
                               "each step moves more than L2: %.2f GB of caches and weights plus "
-                              "the row workspace (GBs)" % (alg["bytes"] / 1e9))},
+                              "the state rows" % (alg["bytes"] / 1e9))},
             "roofline": roof,
             "step_roofline": step_roofline(alg, t_step, peaks, peak_kind, clocks),
             "kernels": {k: {"launches": v[0], "total_ms": round(v[1], 3),

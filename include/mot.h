@@ -212,10 +212,12 @@ mot_status mot_get_schedule(mot_handle h, int32_t* schedule);
  * Per-kernel timing. While enabled, every kernel that translate launches is
  * bracketed by CUDA events on the launching stream. mot_profile_read
  * synchronises those events, writes up to `cap` records (one per kernel
- * name, in first-launch order) and clears the collected events. Backbone
- * handles whose shapes run the window's scan in one launch run its stages one
- * by one while profiling is enabled, so that each has a time of its own; the
- * results agree bit for bit.
+ * name, in first-launch order) and clears the collected events.
+ * enable = 2 brackets the kernels that a call launches otherwise, one after another. enable = 1 is
+ * the same but for backbone handles whose shapes run the window's scan in one
+ * launch: those run its stages one by one, so that each has a time of its own.
+ * The results agree bit for bit. The first enable = 1 on such a handle allocates
+ * the stages' rows, and returns MOT_ERR_OOM (profiling off) where they do not fit.
  */
 typedef struct {
   char name[32];

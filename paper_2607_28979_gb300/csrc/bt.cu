@@ -1,6 +1,6 @@
 // Backbone translators (App. C.2) inside the gated mixture (Def. 3.1) on sm_103a: the gate,
 // the routing, the output projection, and the scan's stages one by one, which run where
-// bt_scan.cu does not take the shapes (and while profiling times them).
+// bt_scan.cu does not take the shapes (and where profiling asks for each).
 //
 // Per token, slot r of the channel window is the source cache entry of layer
 // pi(t_r): P = H_s rows (one per source KV head) of d_s values. A group

@@ -96,8 +96,10 @@ struct BtState {
   // Top-1 routing (token buckets): counts, lists, tile prefixes, packed source rows
   int32_t *rcnt = nullptr, *rlist = nullptr, *rpre = nullptr;
   void* xs = nullptr;   // [G][R][d_s] bf16
-  // the scan in one launch: xo and rstat then hold every slot, and the hidden rows f nothing
+  // the scan in one launch: xo and rstat then hold every slot, and the rows between the staged
+  // kernels (h to xf, f, xs) are allocated when profiling asks for the stages
   bool scan = false;
+  bool staged = false;   // the rows between the staged kernels are allocated
   float* prm = nullptr;   // [G][N] fp32 vectors of the scan
   CUtensorMap tm_wkvh{};
   CUtensorMap tm_win{}, tm_wq{}, tm_wkv{}, tm_wo{}, tm_wf1{}, tm_wf2{}, tm_wout{}, tm_wf1c{};
@@ -184,7 +186,7 @@ struct mot_ctx {
   cudaEvent_t ev_h2d[kHostChunks] = {}, ev_comp[kHostChunks] = {};
   cudaEvent_t ev_prev_compute = nullptr, ev_prev_d2h = nullptr;
   // profiling
-  bool profile = false;
+  int profile = 0;   // 2: every launch as it is otherwise; 1: backbones stage by stage
   std::vector<Ev> ev_used, ev_free;
   std::vector<std::string> kind_names;
   int64_t launches = 0;
@@ -786,6 +788,46 @@ size_t bt_block_elems(const BtDims& d) {
   return size_t(d.E) * d.N * d.Ds + d.E + d.E * expert;
 }
 
+// The rows between the staged kernels, and the tensor maps over them (A operands, boxes of 64 x 128
+// rows): nothing stays allocated where they do not all fit.
+mot_status bt_stage_rows(BtState& bt) {
+  const BtDims& d = bt.d;
+  const size_t G = d.G, R = size_t(d.R), D = d.d, df = d.df;
+  struct A { void** p; size_t n; } rows[] = {
+      {(void**)&bt.h, G * R * D * 4}, {(void**)&bt.ht, G * R * D * 4},
+      {&bt.xz, G * R * D * 2}, {&bt.xq, G * R * D * 2}, {&bt.q, G * R * D * 2},
+      {&bt.kv, G * R * 2 * D * 2}, {&bt.o, G * R * D * 2}, {&bt.xf, G * R * D * 2},
+      {&bt.f, df % 128 ? G * R * df * 2 : 16},
+      {&bt.xs, d.top_k == 1 ? G * R * d.d_s * 2 : 16}};
+  mot_status st = MOT_OK;
+  for (auto& a : rows)
+    if (cudaMalloc(a.p, std::max<size_t>(a.n, 16)) != cudaSuccess) {
+      cudaGetLastError();
+      *a.p = nullptr;
+      st = MOT_ERR_OOM;
+      break;
+    }
+  auto map2 = [&](CUtensorMap* m, void* base, uint64_t inner, uint32_t box_rows) {
+    const uint64_t dims[2] = {inner, G * R};
+    const uint64_t st_b[1] = {inner * 2};
+    const uint32_t box[2] = {64, box_rows};
+    if (st == MOT_OK && !encode_bf16(m, base, 2, dims, st_b, box)) st = MOT_ERR_CUDA;
+  };
+  map2(&bt.tm_xz, bt.xz, D, 128);
+  map2(&bt.tm_xq, bt.xq, D, 128);
+  map2(&bt.tm_o, bt.o, D, 128);
+  map2(&bt.tm_xf, bt.xf, D, 128);
+  if (df % 128) map2(&bt.tm_f, bt.f, df, 128);
+  if (d.top_k == 1) map2(&bt.tm_xs, bt.xs, d.d_s, uint32_t(d.tau * d.P));
+  if (st != MOT_OK)
+    for (auto& a : rows) {
+      if (*a.p) cudaFree(*a.p);
+      *a.p = nullptr;
+    }
+  bt.staged = st == MOT_OK;
+  return st;
+}
+
 mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle* out) {
   if (!out) return MOT_ERR_INVALID_ARG;
   *out = nullptr;
@@ -881,13 +923,8 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
       {&bt.wo, G * N * D * D * 2}, {&bt.wf1, G * N * df * D * 2}, {&bt.wf2, G * N * D * df * 2},
       {&bt.wout, G * bd.Dt * bd.P * D * 2},
       {(void**)&bt.gate, 2 * size_t(bd.B) * bd.S * E * 4},
-      {(void**)&bt.h, G * R * D * 4}, {(void**)&bt.ht, G * R * D * 4},
-      {&bt.xz, G * R * D * 2}, {&bt.xq, G * R * D * 2}, {&bt.q, G * R * D * 2},
-      {&bt.kv, G * R * 2 * D * 2}, {&bt.o, G * R * D * 2}, {&bt.xf, G * R * D * 2},
-      {&bt.f, df % 128 ? G * R * df * 2 : 16},
       {(void**)&bt.rcnt, 64 * 4}, {(void**)&bt.rlist, G * size_t(bd.B) * bd.S * 4},
       {(void**)&bt.rpre, (2 * G + 2) * 4},
-      {&bt.xs, bd.top_k == 1 ? G * R * bd.d_s * 2 : 16},
       {(void**)&h->status, 16}};
   for (auto& a : allocs) {
     if (cudaMalloc(a.p, std::max<size_t>(a.n, 16)) != cudaSuccess) {
@@ -898,7 +935,7 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
     }
   }
   // the scan keeps the state rows of every slot; where they do not fit, those of one slot at
-  // a time and the staged kernels
+  // a time and the staged kernels with their rows
   size_t slots = bt.scan ? N : 1;
   auto state_rows = [&] {
     if (cudaMalloc((void**)&bt.xo, slots * G * R * D * 2) == cudaSuccess &&
@@ -910,14 +947,16 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
     bt.rstat = nullptr;
     return false;
   };
-  if (!state_rows()) {
-    const bool one_slot = slots > 1;
+  if (bt.scan && !state_rows()) {
     bt.scan = false;
     slots = 1;
-    if (!one_slot || !state_rows()) {
+  }
+  if (!bt.scan) {
+    const mot_status staged = state_rows() ? bt_stage_rows(bt) : MOT_ERR_OOM;
+    if (staged != MOT_OK) {
       free_all(h);
       delete h;
-      return MOT_ERR_OOM;
+      return staged;
     }
   }
   if (cudaMemset(h->status, 0, 16) != cudaSuccess || cudaMemset(bt.rcnt, 0, 64 * 4) != cudaSuccess) {
@@ -947,18 +986,12 @@ mot_status bt_create(const mot_config* cfg, const mot_bt_config* bc, mot_handle*
   map2(&bt.tm_wf1c, bt.wf1, D, G * N * df, 128);   // 128-row chunks for the fused FFN
   map2(&bt.tm_wf2, bt.wf2, df, G * N * D, uint32_t(D));
   map2(&bt.tm_wout, bt.wout, uint64_t(bd.P) * D, G * bd.Dt, nt_out);
-  // activations (A operands): box 64 x 128 rows
-  map2(&bt.tm_xz, bt.xz, D, G * R, 128);
-  map2(&bt.tm_xq, bt.xq, D, G * R, 128);
-  map2(&bt.tm_o, bt.o, D, G * R, 128);
-  map2(&bt.tm_xf, bt.xf, D, G * R, 128);
-  if (df % 128) map2(&bt.tm_f, bt.f, df, G * R, 128);
+  // state rows (A operand of the output projection): box 64 x 128 rows
   map2(&bt.tm_xo, bt.xo, uint64_t(bd.P) * D, slots * G * size_t(bd.B) * bd.S, 128);
   if (bd.top_k == 1) {   // Top-1 routing (the default for these handles): token buckets
     uint32_t nt_r = 256;
     while (nt_r > 32 && bd.Dt % nt_r) nt_r -= 32;
     map2(&bt.tm_wout_r, bt.wout, uint64_t(bd.P) * D, G * bd.Dt, nt_r);
-    map2(&bt.tm_xs, bt.xs, bd.d_s, G * R, uint32_t(bd.tau * bd.P));
     h->routing = 1;
   }
   if (!ok) {
@@ -1383,7 +1416,13 @@ mot_status mot_debug_fixed_gate(mot_handle h, const float* gate) {
 
 mot_status mot_profile_enable(mot_handle h, int32_t enable) {
   if (!h) return MOT_ERR_INVALID_ARG;
-  h->profile = enable != 0;
+  h->profile = 0;
+  if (enable != 0 && enable != 2 && h->kind == 2 && !h->bt->staged) {
+    if (cudaSetDevice(h->device) != cudaSuccess) return MOT_ERR_CUDA;
+    const mot_status st = bt_stage_rows(*h->bt);
+    if (st != MOT_OK) return st;
+  }
+  h->profile = enable == 2 ? 2 : enable != 0;
   return MOT_OK;
 }
 
@@ -1525,19 +1564,19 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
       return launch_bt_route(a, bt.rcnt, bt.rlist, bt.rpre, st);
     }));
   }
-  auto project = [&](int r) {   // the output projection of slot r (and the out_slots - 1 after it)
+  auto project = [&](const char* name, int r) {   // slot r's output projection (and out_slots - 1 more)
     a.slot = r;
-    return timed(h, "bt_out_gelu_combine", st, [&] {
+    return timed(h, name, st, [&] {
       return launch_bt_gemm(kBtOut, a, bt.tm_xo, bt.tm_xo, routed ? bt.tm_wout_r : bt.tm_wout,
                             h->num_sms, st);
     });
   };
-  if (bt.scan && !h->profile) {   // profiling times the stages one by one
+  if (bt.scan && h->profile != 1) {   // 1: the stages one by one
     a.prm = bt.prm;
     const CUtensorMap tm[6] = {bt.tm_win, bt.tm_wq, bt.tm_wkvh, bt.tm_wo, bt.tm_wf1c, bt.tm_wf2};
     MOT_CUDA_TRY(timed(h, "bt_scan", st, [&] { return launch_bt_scan(a, tm, h->num_sms, st); }));
     a.out_slots = d.N;
-    MOT_CUDA_TRY(project(0));
+    MOT_CUDA_TRY(project("bt_out_all_slots", 0));
     if (routed) h->counts_valid = true;
     return MOT_OK;
   }
@@ -1571,7 +1610,7 @@ mot_status mot_translate_bt(mot_handle h, const void* src_k, const void* src_v,
         return launch_bt_gemm(kBtF2, a, bt.tm_f, bt.tm_f, bt.tm_wf2, h->num_sms, st);
       }));
     }
-    MOT_CUDA_TRY(project(r));
+    MOT_CUDA_TRY(project("bt_out_gelu_combine", r));
   }
   if (routed) h->counts_valid = true;
   return MOT_OK;

@@ -355,8 +355,14 @@ def mot_debug_set(h: Handle, stall_test: bool, wait_limit_cycles: int = 0) -> No
     _check(_lib.mot_debug_set(h.ptr, int(bool(stall_test)), int(wait_limit_cycles)), "mot_debug_set")
 
 
-def mot_profile_enable(h: Handle, enable: bool = True) -> None:
-    _check(_lib.mot_profile_enable(h.ptr, int(bool(enable))), "mot_profile_enable")
+PROFILE_STAGES, PROFILE_AS_LAUNCHED = 1, 2
+
+
+def mot_profile_enable(h: Handle, enable: int = True) -> None:
+    """True (PROFILE_STAGES): backbone handles run stage by stage; PROFILE_AS_LAUNCHED: every
+    handle's own launches."""
+    level = PROFILE_AS_LAUNCHED if enable is not True and enable == PROFILE_AS_LAUNCHED else int(bool(enable))
+    _check(_lib.mot_profile_enable(h.ptr, level), "mot_profile_enable")
 
 
 def mot_profile_read(h: Handle) -> dict:

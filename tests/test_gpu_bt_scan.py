@@ -1,6 +1,6 @@
 """The backbone translators' scan in one launch, at the edges of its tiles, chunks and
 attention blocks: against the fp64 oracle, and against the staged schedule (which runs
-while profiling is enabled) for what must agree bit for bit or position by position."""
+while profiling of the stages is enabled) bit for bit."""
 import numpy as np
 import pytest
 
@@ -127,23 +127,29 @@ def test_scan_keeps_non_finite_tokens_apart():
 
 
 def test_no_room_for_every_slot_runs_the_staged_kernels():
-    """Where the state rows of all slots (519 MB here) do not fit but those of one slot do
-    (410 MB of workspace in all), the handle is created all the same and a call runs the staged
+    """Where the state rows of all slots (553 MB here) do not fit but those of one slot and of the stages
+    do (about 440 MB with the weights), the handle is created all the same and a call runs the staged
     schedule: its launches, and its output bit for bit."""
     lens = (40, 7)
     wl = W("bt_room", 1, 16, 64, 16, 2, 32, 2, 0, 2, 1024, "bf16", lens, bt=(0, 16, 128, 4, 128))
     sk, sv, blob = _inputs(wl, 11)
     want = _run(wl, sk, sv, blob, staged=True)
-    torch.cuda.synchronize()
-    torch.cuda.empty_cache()
-    h = M.mot_create_bt(*M.bt_config_from(wl))
-    M.mot_destroy(h)
     k, v = G.to_device(wl, sk), G.to_device(wl, sv)
     (_, dk), (_, dv) = G.alloc_dst(wl), G.alloc_dst(wl)
     lens_d = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
     free = torch.cuda.mem_get_info()[0]
-    held = torch.empty(free - (720 << 20), dtype=torch.uint8, device="cuda")
-    h = M.mot_create_bt(*M.bt_config_from(wl))
+    held = torch.empty(free - (500 << 20), dtype=torch.uint8, device="cuda")
+    left = torch.cuda.mem_get_info()[0]
+    if not 480 << 20 < left < 520 << 20:
+        pytest.skip("the GPU's memory is in use elsewhere")
+    try:
+        h = M.mot_create_bt(*M.bt_config_from(wl))
+    except M.MotError:
+        if torch.cuda.mem_get_info()[0] < left - (8 << 20):
+            pytest.skip("the GPU's memory is in use elsewhere")
+        raise
     del held
     torch.cuda.empty_cache()
     M.mot_load_weights(h, blob)
@@ -153,6 +159,41 @@ def test_no_room_for_every_slot_runs_the_staged_kernels():
     assert M.mot_get_launch_count(h) - c0 == want[2]
     assert torch.equal(G.int_view(dk), G.int_view(want[0]))
     assert torch.equal(G.int_view(dv), G.int_view(want[1]))
+
+
+@pytest.mark.parametrize("top_k", [0, 1])
+def test_profile_of_the_launches_and_of_the_stages(top_k):
+    """Profiling as launched times the kernels that an ordinary call runs; the stages' rows are only
+    there once their times are asked for."""
+    wl = W("bt_prof", 2, 16, 64, 2, 2, 32, 2, 0, 2, 1024, "bf16", (40, 7), top_k=top_k, bt=(0, 2, 128, 4, 128))
+    sk, sv, blob = _inputs(wl, 17)
+    want = _run(wl, sk, sv, blob)
+    torch.cuda.synchronize()
+    k, v = G.to_device(wl, sk), G.to_device(wl, sv)
+    lens = torch.tensor(wl.seq_lens, dtype=torch.int32, device="cuda")
+    (_, dk), (_, dv) = G.alloc_dst(wl), G.alloc_dst(wl)
+    rows = 2 * wl.n_translators * 2 * 1024 * 16        # [K/V][E][B][S][P]
+    free = torch.cuda.mem_get_info()[0]
+    h = M.mot_create_bt(*M.bt_config_from(wl))
+    M.mot_load_weights(h, blob)
+    used = free - torch.cuda.mem_get_info()[0]
+    assert used < rows * 2 * (2 * 128 + 8) + (64 << 20)   # state rows and statistics of both slots
+    for level, names in ((M.PROFILE_AS_LAUNCHED, {"bt_gate", "bt_scan", "bt_out_all_slots"}),
+                         (M.PROFILE_STAGES, {"bt_gate", "bt_in_ln_gelu", "bt_q", "bt_kv", "bt_attn",
+                                             "bt_o_residual_ln", "bt_ffn_fused", "bt_out_gelu_combine"})):
+        M.mot_profile_enable(h, level)
+        c0 = M.mot_get_launch_count(h)
+        M.mot_translate_bt(h, k, v, lens, wl.batch, dk, dv)
+        prof = M.mot_profile_read(h)
+        routed = {"bt_route"} | ({"bt_pack"} if level == M.PROFILE_STAGES else set()) if top_k else set()
+        assert {n for n, (launches, _) in prof.items() if launches} == names | routed
+        assert sum(launches for launches, _ in prof.values()) == M.mot_get_launch_count(h) - c0
+        if level == M.PROFILE_AS_LAUNCHED:
+            assert M.mot_get_launch_count(h) - c0 == want[2]
+        assert torch.equal(G.int_view(dk), G.int_view(want[0]))
+        assert torch.equal(G.int_view(dv), G.int_view(want[1]))
+    assert free - torch.cuda.mem_get_info()[0] > used + rows * 128 * 20
+    M.mot_destroy(h)
 
 
 @pytest.mark.parametrize("top_k", [0, 1])

@@ -80,8 +80,7 @@ def _load(buf, draw):
 def test_chain_captured_and_back_to_back(name):
     h, draws, buf, out, call = _chain(name)
     st = torch.cuda.Stream()
-    # backbones run other kernels while profiling: they are compared with separate calls
-    M.mot_profile_enable(h, name != "backbones")
+    M.mot_profile_enable(h, M.PROFILE_AS_LAUNCHED)
     want = []
     with torch.cuda.stream(st):
         for d in draws:
