@@ -170,7 +170,8 @@ __global__ void __launch_bounds__(32 * Rg<D, NT>::kWarps, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int G = d.Hq / d.Hkv;
-  if (a.stall_test && blockIdx.x == 0) {   // test hook: wait (bounded) for a signal nothing sends
+  if (a.stall_test && blockIdx.x == 0) {   // test hook for the report of a timeout: the kernel waits for
+    // nothing but its own copies, so this is a bounded wait of the hook's own
     __shared__ uint64_t never;
     __shared__ int gave_up;
     if (threadIdx.x == 0) {

@@ -280,10 +280,12 @@ def test_batch_prefix_and_errors():
 
 
 def test_guided_timeout_is_reported_and_recovers():
-    """Failure detection without a fault: with the stall hook the guided kernel's
-    first CTA withholds one MMA completion signal, its wait runs out after the
-    short limit, the kernel unwinds and the status word reports a timeout. The
-    next guided layer on the same context matches the oracle."""
+    """Failure reporting without a fault: with the stall hook the guided kernel's
+    first CTA waits for a signal that nothing sends, the wait runs out after the
+    short limit, the CTA leaves and the status word reports a timeout. (The kernel
+    itself waits for its own copies only, so this covers the report and the next
+    call, not an unwinding pipeline.) The next guided layer on the same context
+    matches the oracle."""
     wl = SMALL["r_gqa6_d128"]
     q, k, v = synth.gen_replay_qkv(wl, 3)
     g = synth.gen_guide(wl, 6)
