@@ -462,3 +462,34 @@ def test_infinities_and_nans(d, group, top_s, n):
                         assert (raw[:, u][fin] == clean[:, u][fin]).all(), u
                     elif fin.any():
                         G.assert_parity(BF16, x[fin], ref[fin], f"layer {layer} u {u}")
+
+
+@pytest.mark.parametrize("kv,lens", [(5, (40, 0, 33)), (2, (40, 1, 17, 40)), (4, tuple(1 + 13 * b % 40 for b in range(30))),
+                                     (7, tuple(40 - b % 3 for b in range(64)))])
+@pytest.mark.parametrize("top_s", [24, 130])
+def test_every_item_of_ragged_batches(kv, lens, top_s):
+    """Items walk over positions and heads in passes of the grid's warps: whole positions, turning to
+    the next head with each pass, or (many heads) any part of one. Every row inside its sequence, and
+    no other, against numpy."""
+    import _helpers as H
+    n = 41
+    wl = RW("r_items", 2, 3, kv, kv, 64, len(lens), n, lens, top_s=top_s, n_full=1)
+    q, k, v = synth.gen_replay_qkv(wl, 53)
+    g = synth.gen_guide(wl, 59)
+    run = ReplayRun(wl)
+    sel = run.select(g)
+    qd, kd, vd = (H.bf16_bits_to_f64(x) for x in (q, k, v))
+    for layer in (0, 2):
+        out = run.attend(layer, q, k, v, None if layer == 0 else g)
+        got, raw = _f64(out), out.cpu().numpy()
+        s = np.einsum("bhud,bhjd->bhuj", qd, kd) / 8.0
+        ref = np.zeros_like(got)
+        for b, L in enumerate(lens):
+            assert (raw[b, :, L:] == np.int16(G.SENTINEL_BF16)).all()
+            for u in range(L):
+                at = np.arange(u + 1) if layer == 0 else sel[b, u][sel[b, u] >= 0]
+                p = np.exp(s[b, :, u, at] - s[b, :, u, at].max(0))
+                ref[b, :, u] = np.einsum("jh,hjd->hd", p / p.sum(0), vd[b][:, at])
+        inside = np.arange(n)[None] < np.array(lens)[:, None]
+        rows = np.broadcast_to(inside[:, None], got.shape[:3])
+        G.assert_parity(BF16, got[rows], ref[rows], f"layer {layer}")
