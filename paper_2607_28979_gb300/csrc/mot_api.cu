@@ -1683,7 +1683,7 @@ mot_status replay_args(mot_handle h, const void* q, const void* k, const void* v
   a.out = out;
   a.sel = h->rsel;
   a.sel_stride = sel_row(d);
-  a.pad_first = 1;
+  a.pad = 1;
   a.seq_lens = seq_lens;
   a.batch = batch;
   a.status = h->status;
@@ -1705,7 +1705,7 @@ mot_status mot_replay_select(mot_handle h, const void* guide, const int32_t* seq
   if (batch == 0) return MOT_OK;
   a.sel = sel;
   a.sel_stride = h->rd.S;
-  a.pad_first = 0;
+  a.pad = 0;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   MOT_CUDA_TRY(timed(h, "replay_select", st, [&] { return launch_replay_select(a, h->num_sms, st); }));
   return MOT_OK;

@@ -81,14 +81,20 @@ __device__ __forceinline__ uint32_t ord16x2(uint32_t q) {
   return q ^ (sign | 0x80008000u);
 }
 
-// A full row of S entries in a workspace of wider rows: the rest repeats its first position.
-__device__ __forceinline__ void pad_row(const ReplayArgs& a, int32_t* out) {
-  const int lane = threadIdx.x & 31;
-  if (a.sel_stride > a.d.S) {
+// A workspace row's entries past its positions repeat them in turn: were they all one position (the
+// first, which many rows hold), the gathers of a set of 100 in 128 slots would queue at its L2 slice
+// (4 x 4096 positions, 12 heads of 128 on 2, S = 70: 307 us, 142 so; also rows below S, where all the
+// padding was position 0: 100 positions, 28 heads on 4, S = 128: 21 us, 11 so).
+__device__ __forceinline__ void pad_row(const ReplayArgs& a, int32_t* out) {   // S positions found
+  const int lane = threadIdx.x & 31, S = a.d.S;
+  if (a.sel_stride > S) {
     __syncwarp();
-    const int32_t first = *static_cast<volatile int32_t*>(out);
-    for (int j = a.d.S + lane; j < a.sel_stride; j += 32) out[j] = first;
+    for (int j = S + lane; j < a.sel_stride; j += 32)
+      out[j] = static_cast<volatile int32_t*>(out)[(j - S) % S];
   }
+}
+__device__ __forceinline__ void take_all(const ReplayArgs& a, int32_t* out, int n) {   // n <= S positions
+  for (int j = threadIdx.x & 31; j < a.sel_stride; j += 32) out[j] = j < n ? j : a.pad ? j % n : -1;
 }
 
 // Selection for any max_seq. One warp per context row (b, u). With o = the
@@ -110,7 +116,7 @@ __global__ void __launch_bounds__(32 * kSelWarps) replay_select_stream_kernel(co
   int32_t* out = a.sel + int64_t(row) * a.sel_stride;
   const int n = u + 1;
   if (n <= d.S) {
-    for (int j = lane; j < a.sel_stride; j += 32) out[j] = j < n ? j : a.pad_first ? 0 : -1;
+    take_all(a, out, n);
     return;
   }
   const uint16_t* A = static_cast<const uint16_t*>(a.guide) + int64_t(row) * d.N;
@@ -219,7 +225,7 @@ __global__ void __launch_bounds__(32 * kSelCacheWarps) replay_select_hist_kernel
   int32_t* out = a.sel + int64_t(row) * a.sel_stride;
   const int n = u + 1;
   if (n <= d.S) {
-    for (int j = lane; j < a.sel_stride; j += 32) out[j] = j < n ? j : a.pad_first ? 0 : -1;
+    take_all(a, out, n);
     return;
   }
   const uint16_t* A = static_cast<const uint16_t*>(a.guide) + int64_t(row) * d.N;
@@ -742,7 +748,7 @@ __global__ void __launch_bounds__(32 * kSelRowWarps, kSelRowCtas)
     int32_t* out = a.sel + int64_t(row) * a.sel_stride;
     const int n = u + 1;
     if (n <= d.S) {
-      for (int j = lane; j < a.sel_stride; j += 32) out[j] = j < n ? j : a.pad_first ? 0 : -1;
+      take_all(a, out, n);
       continue;
     }
     const RowWords rw(a, row, n);

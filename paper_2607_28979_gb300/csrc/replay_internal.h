@@ -25,7 +25,7 @@ struct ReplayArgs {
   void* out;
   int32_t* sel;
   int64_t sel_stride;     // entries from one row of sel to the next
-  int32_t pad_first;      // fill a row's unused entries with its first position (else -1)
+  int32_t pad;            // a row's unused entries repeat its positions (else -1)
   const int32_t* seq_lens;
   int32_t batch;
   int32_t full;   // 1: attend to every position 0..u
@@ -44,7 +44,7 @@ cudaError_t launch_replay_fmha(const ReplayArgs& a, const CUtensorMap& tmK,
                                const CUtensorMap& tmVt, cudaStream_t st);
 cudaError_t launch_replay_select(const ReplayArgs& a, int num_sms, cudaStream_t st);
 // Guided layers, and full layers that launch_replay_fmha does not take. The rows of a.sel are
-// whole units of replay_gather_unit(d) entries, the unused ones filled (pad_first) with a
+// whole units of replay_gather_unit(d) entries, the unused ones filled (pad) with a
 // position of the set. Persistent, one CTA per SM.
 int replay_gather_unit(const ReplayDims& d);
 cudaError_t launch_replay_gather(const ReplayArgs& a, int num_sms, cudaStream_t st);
