@@ -10,7 +10,7 @@
 //                         bisection over those gives the threshold V and how many of
 //                         the positions scoring V are taken. Rows with u + 1 <= S take
 //                         every position.
-//   replay_select_hist_kernel, for S past 448: the threshold from two histograms over
+//   replay_select_hist_kernel, for S past 416: the threshold from two histograms over
 //                         the row's keys in shared memory.
 //   replay_select_stream_kernel, for rows past 4,096 positions: histograms of the high
 //                         and the low byte, reading the row once per pass.
@@ -443,7 +443,8 @@ constexpr int kSelRowWarps = 4;
 constexpr int kSelRowCtas = 10;      // CTAs per SM (up to 51 registers a thread)
 constexpr int kSelRowSeq = 4096;     // largest max_seq taken
 constexpr int kSelOneSet = 160;      // largest S taken with 256 group maxima
-constexpr int kSelTwoSets = 448;     // largest S taken with 512
+constexpr int kSelTwoSets = 416;     // largest S taken with 512: four rows of 4,096, S = 416: 66 us (75 by
+                                     // histograms), 432: 79 (75), 448: 97 (74); of 1,024: equal
 
 // Keys of packed pairs against a threshold key. RAW keys are non-negative bf16 bits below the
 // NaNs, which order as the numbers they are: one packed comparison per pair.

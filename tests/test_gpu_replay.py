@@ -340,10 +340,10 @@ def test_gathered_rows_every_unit_size(d, group, top_s, n):
 
 
 @pytest.mark.parametrize("max_seq", [257, 263, 520, 1030, 2049, 4093])   # every 16-byte phase of a row start
-@pytest.mark.parametrize("top_s", [1, 128, 160, 161, 256, 449])
+@pytest.mark.parametrize("top_s", [1, 128, 160, 161, 256, 416, 417, 449])
 def test_selection_bounds_lists_and_fallback(max_seq, top_s):
     """The bounded selection against numpy, bit for bit: one or two sets of group maxima
-    (top_s up to 160 and 448) and the histogram past them; rows whose candidates overflow
+    (top_s up to 160 and 416) and the histogram past them; rows whose candidates overflow
     the list (a few values only), rows of distinct scores, mixed signs, and rows holding the
     lowest key (a negative NaN pattern), whose bound cannot separate it from empty slots."""
     wl = RW("r_bound", 2, 2, 1, 1, 64, 2, max_seq, (max_seq, max_seq - 3), top_s=top_s, n_full=1)
