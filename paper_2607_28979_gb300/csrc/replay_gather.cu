@@ -13,7 +13,7 @@
 //                         own copy groups.
 //
 // What bounds it: the gathers, S * 2 * d * 2 bytes per item out of L2 (2.15 GB for
-// 4 x 4096 positions, 2 key/value heads, d = 128, S = 128; 15 TB/s, L2-to-SM links 54%
+// 4 x 4096 positions, 2 key/value heads, d = 128, S = 128; 15.6 TB/s, L2-to-SM links 54%
 // busy on average and 64% on the busiest slice). Why warps on mma.sync and not the
 // fifth-generation tensor cores: the products are small (heads x S x d), and a tcgen05
 // item needs a lane of four warps with 72 KB of tiles, four barriers and two serial MMA
@@ -22,16 +22,17 @@
 // 252 us as three tcgen05 lanes, 248 us with the MMA fragments loaded straight from global
 // memory (each 16-byte load instruction touches 4 to 8 rows: 1,650 L1 wavefronts per item),
 // 177 us with this ring and a general tile cursor (3,200 instructions per item), 162 us
-// with the static tile stream (1,550), 142 to 151 us with the item and tile orders below (by run).
+// with the static tile stream (1,550), 142 to 151 us with the tile orders below, 140 us with the
+// item order below and the selection's spare slots spread (pad_row in replay.cu).
 //
 // Probabilities that the CUDA-core kernel before this one held in fp32 (heads of 64, sets past
 // 128 rows, full layers) stay fp32: three bf16 parts, exact. Two parts rounded to 2^-17 moved the
 // error against 64 bits from 1.630332e-3 to 1.630333e-3; with three it is the
 // former kernel's to eight digits, with the small parts added apart from the large one where they
-// take MMAs of their own (three sums into one accumulator over 1,500 rows: + 2e-10). Whole calls,
-// CUDA cores, two parts, three: 8 x 1024 positions, 12 heads of 64, S = 128: 739, 227, 227 us;
-// 4 x 4096, 12 heads of 128 on 2, S = 256: 296 and 328 us (1,127 us for the former kernel alone); full causal
-// layers of 2047 + 1025 positions, the same heads: 231 and 279 us (980).
+// take MMAs of their own (three sums into one accumulator over 1,500 rows: + 2e-10). The time on
+// CUDA cores, with two parts, and with three and today's order of items: 8 x 1024 positions, 12
+// heads of 64, S = 128: 691, 213, 204 us; 4 x 4096, 12 heads of 128 on 2, S = 256: 1,127, 248, 279
+// us; full causal layers of 2047 + 1025 positions, the same heads: 984, 232, 259 us.
 #include "replay_common.cuh"
 
 namespace mot {
