@@ -231,18 +231,21 @@ struct Attn {
   static constexpr int NA = kScD / DH, CH = DH / 8;   // heads; 16-byte pieces of one
   static constexpr int NR = DH <= 32 ? 2 : 1;         // rows of a thread
 };
-struct AttnTask {   // rows p and p + ceil(P / NR) of a token (its first row rb), the head's first piece
+struct AttnTask {   // rows p and p + ceil(P / NR), if it has one, of a token (first row rb); the head's first piece
   int rb, r[2], blk, c0;
-  bool two;         // the second row is one of its own
+  bool two;         // the second row is another one than the first
 };
+// Lanes past the tile's last task repeat it: no lane reads query rows that another warp overwrites.
 template <int DH>
 __device__ __forceinline__ AttnTask attn_task(int task, int P, int tau) {
   using A = Attn<DH>;
   const int per = (P + A::NR - 1) / A::NR;
+  task = min(task, tau * A::NA * per - 1);
   const int th = task / per, p0 = task - th * per;
-  const int tok = min(th / A::NA, tau - 1), hd = th % A::NA;
-  const int rb = tok * P, p1 = min(p0 + per, P - 1);
-  return {rb, {rb + p0, rb + p1}, ((hd * A::CH) >> 3) * kScBlk, (hd * A::CH) & 7, p0 + per < P};
+  const int tok = th / A::NA, hd = th - tok * A::NA;
+  const int rb = tok * P;
+  const bool two = p0 + per < P;
+  return {rb, {rb + p0, rb + p0 + (two ? per : 0)}, ((hd * A::CH) >> 3) * kScBlk, (hd * A::CH) & 7, two};
 }
 template <int DH>
 __device__ __forceinline__ void attend(uint8_t* qt, const uint8_t* kt, const uint8_t* vt, uint32_t scratch,
